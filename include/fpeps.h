@@ -54,13 +54,15 @@ typedef enum {
 
 /* Arithmetic of the contraction GEMMs (the QR and the small SVD always run in
  * FP64-class precision). FP64: everything in double. F32: plain FP32 CUDA-core
- * products. TF32X3 / BF16X3: split-precision products on the tensor cores,
- * a_hi*b_hi + a_hi*b_lo + a_lo*b_hi with FP32 accumulation, the operands split
- * into TF32 (3 x 2^-22 relative error per product) or BF16 (3 x 2^-16) halves.
- * In BF16X3 every tensor-core GEMM (boundary and environment products, the
- * QR's tall products, the CBE projectors) takes the BF16 split; the site
- * sandwich stays 3xTF32, and the calibration columns and unbiased products
- * run on the FP32 CUDA cores as in TF32X3. */
+ * products. TF32X3: split-precision products on the tensor cores,
+ * a_hi*b_hi + a_hi*b_lo + a_lo*b_hi with FP32 accumulation, every operand split
+ * into two 11-bit halves (3 x 2^-22 relative error per product). Small products
+ * split into TF32 halves on chip; large ones into FP16 halves with a power-of-two
+ * scale per row and 256 terms, where an element more than 2^18 below the largest
+ * of its row and 256 terms keeps 2^-40 of that largest instead. BF16X3 (two
+ * 8-bit halves, 3 x 2^-16) is at most as accurate as that and no faster, so a
+ * BF16X3 environment runs the same products. The site sandwich is 3xTF32, and the
+ * calibration columns and unbiased products run on the FP32 CUDA cores. */
 typedef enum { FPEPS_F64 = 0, FPEPS_F32 = 1, FPEPS_TF32X3 = 2, FPEPS_BF16X3 = 3 } fpeps_precision;
 
 /* Device-memory provider. alloc(ctx, bytes, stream) returns device memory usable

@@ -1,8 +1,10 @@
 // C ABI of libfpeps: environment lifecycle, the row state machine and
 // checkpoints. Every entry point converts internal errors to fpeps_status.
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <mutex>
+#include <map>
 #include <cstring>
 #include <exception>
 #include <new>
@@ -13,14 +15,57 @@ using fpeps::Error;
 
 namespace fpeps {
 
+// Scratch of the calls without a handle (fpeps_gemm_f32): a pool of the library's own per device,
+// shared by all threads and streams (stream-ordered). The default pool hands its memory back at
+// every synchronisation, and mapping half a gigabyte again costs the next call a millisecond; this
+// one keeps up to kKeep bytes, which trim_pools() gives back (when an environment is destroyed or an
+// allocation fails).
+namespace {
+constexpr uint64_t kKeep = 640ull << 20;
+std::mutex g_pool_mu;
+std::map<int, cudaMemPool_t> g_pools;
+}  // namespace
+
+static cudaMemPool_t scratch_pool() {
+  int dev = 0;
+  FP_CUDA(cudaGetDevice(&dev));
+  std::lock_guard<std::mutex> lk(g_pool_mu);
+  auto it = g_pools.find(dev);
+  if (it != g_pools.end()) return it->second;
+  cudaMemPoolProps pr = {};
+  pr.allocType = cudaMemAllocationTypePinned;
+  pr.location.type = cudaMemLocationTypeDevice;
+  pr.location.id = dev;
+  cudaMemPool_t pool;
+  FP_CUDA(cudaMemPoolCreate(&pool, &pr));
+  uint64_t keep = kKeep;
+  FP_CUDA(cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep));
+  g_pools[dev] = pool;
+  return pool;
+}
+
+static void trim_pools() {
+  std::lock_guard<std::mutex> lk(g_pool_mu);
+  for (auto& p : g_pools) cudaMemPoolTrimTo(p.second, 0);
+}
+
 void* Allocator::get(size_t bytes) {
   void* p = nullptr;
   if (has) {
     p = a.alloc(a.ctx, bytes, (void*)stream);
+    if (!p) {
+      trim_pools();
+      p = a.alloc(a.ctx, bytes, (void*)stream);
+    }
     if (!p) throw Error{FPEPS_ERR_OOM, "allocator returned NULL for " + std::to_string(bytes) + " bytes"};
     return p;
   }
   cudaError_t e = cudaMallocAsync(&p, bytes, stream);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    trim_pools();
+    e = cudaMallocAsync(&p, bytes, stream);
+  }
   if (e == cudaErrorMemoryAllocation) {
     cudaGetLastError();
     throw Error{FPEPS_ERR_OOM, "cudaMallocAsync failed for " + std::to_string(bytes) + " bytes"};
@@ -589,6 +634,7 @@ void fpeps_env_destroy(fpeps_env* env) {
     if (env->stream || !env->al.has) cudaStreamSynchronize(env->stream);
     if (env->h_info) cudaFreeHost(env->h_info);
     if (env->h_scal) cudaFreeHost(env->h_scal);
+    fpeps::trim_pools();
   } catch (...) {
   }
   delete env;
@@ -642,12 +688,12 @@ fpeps_status fpeps_apply_theta_op(fpeps_env* env, int32_t op, int32_t c, int32_t
 fpeps_status fpeps_selftest_wait_timeout(void* cuda_stream) {
   return fpeps::guard(nullptr, [&] {
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    // a 128-row product runs on a single CTA, a 256-row one on a CTA pair
+    // both kernels, a 128-row product (a single CTA) and a 256-row one (a CTA pair)
     int timed_out = 0;
-    for (const int64_t M : {128, 256}) {
-      const int64_t N = 128, K = 32;
+    for (int t = 0; t < 4; ++t) {
+      const int64_t M = t % 2 ? 256 : 128, N = 128, K = 32;
       float *A = nullptr, *B = nullptr, *C = nullptr;
-      const size_t sb = fpeps::gemm_tc_scratch_bytes(FPEPS_TF32X3, M, N, K);
+      const size_t sb = std::max<size_t>(fpeps::gemm_onchip_scratch_bytes(M, N, K), 256);
       int* err = nullptr;
       FP_CUDA(cudaMallocAsync((void**)&A, sizeof(float) * M * K, s));
       FP_CUDA(cudaMallocAsync((void**)&B, sizeof(float) * N * K, s));
@@ -656,7 +702,8 @@ fpeps_status fpeps_selftest_wait_timeout(void* cuda_stream) {
       FP_CUDA(cudaMemsetAsync(A, 0, sizeof(float) * M * K, s));
       FP_CUDA(cudaMemsetAsync(B, 0, sizeof(float) * N * K, s));
       FP_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
-      fpeps::gemm_tc(s, FPEPS_TF32X3, M, N, K, A, K, B, K, C, fpeps::out_rowmajor(M, N, N), err, sb, true);
+      if (t < 2) fpeps::gemm_onchip(s, M, N, K, A, K, B, K, C, fpeps::out_rowmajor(M, N, N), err, sb, true);
+      else fpeps::gemm_tc_hold(s, M, N, K, A, C, err);
       int h = 0;
       FP_CUDA(cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, s));
       FP_CUDA(cudaStreamSynchronize(s));
@@ -667,7 +714,7 @@ fpeps_status fpeps_selftest_wait_timeout(void* cuda_stream) {
       FP_CUDA(cudaStreamSynchronize(s));
       timed_out += h != 0;
     }
-    if (timed_out == 2) throw Error{FPEPS_ERR_TIMEOUT, "tensor-core GEMM: bounded waits ran out as designed"};
+    if (timed_out == 4) throw Error{FPEPS_ERR_TIMEOUT, "tensor-core GEMM: bounded waits ran out as designed"};
   });
 }
 
@@ -684,11 +731,11 @@ fpeps_status fpeps_gemm_f32(int32_t mode, int64_t M, int64_t N, int64_t K, const
     if (mode != FPEPS_TF32X3 && mode != FPEPS_BF16X3) throw Error{FPEPS_ERR_UNSUPPORTED, "mode"};
     if (!fpeps::gemm_tc_supported(M, N, K, lda, ldb) || ((uintptr_t)A % 16) || ((uintptr_t)B % 16))
       throw Error{FPEPS_ERR_UNSUPPORTED, "shape not supported by the tensor-core kernel"};
-    const size_t sb = fpeps::gemm_tc_scratch_bytes(mode, M, N, K);
+    const size_t sb = fpeps::gemm_tc_scratch_bytes(M, N, K);
     int* err = nullptr;
-    FP_CUDA(cudaMallocAsync((void**)&err, sb, s));
+    FP_CUDA(cudaMallocFromPoolAsync((void**)&err, sb, fpeps::scratch_pool(), s));
     FP_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
-    fpeps::gemm_tc(s, mode, M, N, K, A, lda, B, ldb, C, om, err, sb);
+    fpeps::gemm_tc(s, M, N, K, A, lda, B, ldb, C, om, err, sb);
     int h = 0;
     FP_CUDA(cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, s));
     FP_CUDA(cudaStreamSynchronize(s));

@@ -93,14 +93,26 @@ template <class T>
 void gemm_simt(cudaStream_t s, int64_t M, int64_t N, int64_t K, T alpha, const T* A, int64_t a_m,
                int64_t a_k, const T* B, int64_t b_n, int64_t b_k, T beta, T* C, OutMap om);
 
-// Tensor-core GEMM for K-major A [M][lda] and B [N][ldb] (k contiguous), split
-// precision (mode 2 = 3xTF32, 3 = 3xBF16). Returns false if the shape is not
-// supported by the tensor-core path (caller falls back to nothing: it is an error).
+// Tensor-core GEMM for K-major A [M][lda] and B [N][ldb] (k contiguous), every operand split
+// into two 11-bit halves: products that amortise it run on FP16 planes made beforehand (gemm_tc.cu),
+// the others split into TF32 on chip (gemm_onchip.cu). scratch: its first int is the
+// error word (set to 1 when a bounded wait timed out).
 bool gemm_tc_supported(int64_t M, int64_t N, int64_t K, int64_t lda, int64_t ldb);
-void gemm_tc(cudaStream_t s, int mode, int64_t M, int64_t N, int64_t K, const float* A, int64_t lda,
-             const float* B, int64_t ldb, float* C, OutMap om, void* scratch, size_t scratch_bytes,
-             bool hold_loads = false);   // hold_loads: self-test of the bounded waits (no loads issued)
-size_t gemm_tc_scratch_bytes(int mode, int64_t M, int64_t N, int64_t K);
+void gemm_tc(cudaStream_t s, int64_t M, int64_t N, int64_t K, const float* A, int64_t lda, const float* B,
+             int64_t ldb, float* C, OutMap om, void* scratch, size_t scratch_bytes);
+size_t gemm_tc_scratch_bytes(int64_t M, int64_t N, int64_t K);
+void gemm_onchip(cudaStream_t s, int64_t M, int64_t N, int64_t K, const float* A, int64_t lda, const float* B, int64_t ldb, float* C, OutMap om, void* scratch, size_t scratch_bytes,
+                 bool hold_loads = false);   // hold_loads: self-test of the bounded waits (no loads issued)
+size_t gemm_onchip_scratch_bytes(int64_t M, int64_t N, int64_t K);
+// a split operand: planes [rows][k-blocks of 32 terms][32 hi, 32 lo halves], 2^-e of row r in the
+// chunk c of 256 terms at inv[c * inv_stride + r]
+struct SplitMat {
+  const void* planes;
+  const float* inv;
+  int64_t inv_stride;
+};
+// self-test of the bounded waits of the planes kernel (no loads issued); planes: any device memory
+void gemm_tc_hold(cudaStream_t s, int64_t M, int64_t N, int64_t K, void* planes, float* C, void* scratch);
 
 // ---------------------------------------------------------------- sandwich
 // Bundle order. A (ket, PEPO, bra) bundle of dims (n, nw, n) is indexed (x nw + x_w) n + x'

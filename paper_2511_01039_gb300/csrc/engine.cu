@@ -204,7 +204,7 @@ struct Engine : EngineBase {
     if (sizeof(T) == 4 && (mode == FPEPS_TF32X3 || mode == FPEPS_BF16X3) && !simt_only &&
         gemm_tc_supported(M, N, K, lda, ldb) &&
         ((uintptr_t)A % 16) == 0 && ((uintptr_t)B % 16) == 0) {
-      size_t need = gemm_tc_scratch_bytes(mode, M, N, K);
+      size_t need = gemm_tc_scratch_bytes(M, N, K);
       if (!tc_scr || tc_n < need) {
         if (tc_scr) {
           check_tc();   // keep a recorded timeout before the error word is replaced
@@ -214,7 +214,7 @@ struct Engine : EngineBase {
         tc_n = std::max<size_t>(need, 256);
         FP_CUDA(cudaMemsetAsync(tc_scr, 0, sizeof(int), s));
       }
-      gemm_tc(s, mode, M, N, K, (const float*)A, lda, (const float*)B, ldb, (float*)C, om, tc_scr, tc_n);
+      gemm_tc(s, M, N, K, (const float*)A, lda, (const float*)B, ldb, (float*)C, om, tc_scr, tc_n);
       tc_used = true;
       return;
     }

@@ -135,15 +135,6 @@ __device__ __forceinline__ void mma_ts(uint32_t d, uint32_t a, uint64_t b, uint3
       : "memory");
 }
 
-// waits for this thread's tensor-memory loads, then ties the loaded registers to the wait so
-// that no use of them is scheduled before it
-template <int N>
-__device__ __forceinline__ void tmem_wait_tie(uint32_t (&r)[N]) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < N; ++i) asm volatile("" : "+r"(r[i]));
-}
-
 __device__ __forceinline__ void named_sync(int id, int n) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
