@@ -338,10 +338,11 @@ fpeps_status fpeps_gemm_f32(int32_t mode, int64_t M, int64_t N, int64_t K, const
  * descending and U, V column-major k x k (device). Columns whose singular value
  * is below 1e-15 of the Frobenius norm get a zero U column. 1 <= k <= 1024.
  * The path passes the transposed triangular factor of a QR, for which the
- * method converges in about ten sweeps; the sweep count is capped at 30, so a
- * badly conditioned general matrix may return before full convergence.
- * Allocates its scratch (2 k^2 doubles) with cudaMallocAsync on `cuda_stream`
- * and synchronises it. */
+ * method converges in about ten sweeps (most of them in FP32, then corrected and
+ * checked in FP64); the sweep count is capped at 30, so a badly conditioned
+ * general matrix may return before full convergence.
+ * Takes its scratch (about 5.5 k^2 doubles) stream-ordered on `cuda_stream` from a
+ * pool of the library, and synchronises the stream. */
 fpeps_status fpeps_svd_f64(const double* M, int32_t k, double* U, double* sigma, double* V, void* cuda_stream);
 
 /* Largest k accepted by fpeps_svd_f64_noalloc. */
@@ -350,8 +351,8 @@ fpeps_status fpeps_svd_f64(const double* M, int32_t k, double* U, double* sigma,
 /* Same SVD as fpeps_svd_f64, for callers that cannot allocate device memory
  * during the call (for instance when another allocator already owns the whole
  * device pool, or in a latency-critical loop where an allocation could stall or
- * fail). It allocates nothing: its working storage (2 k^2 doubles, k ints and a
- * few counters; about 1.05 MB) is a fixed device array inside the library, held
+ * fail). It allocates nothing: its working storage (5 k^2 doubles, k^2 floats
+ * and some lists; about 3 MB) is a fixed device array inside the library, held
  * on every GPU that loads the library until the process exits. The paper has no
  * counterpart; this is an interface of this library only.
  *   M (k x k, column-major, device, unchanged), U, V (k x k, column-major,

@@ -91,7 +91,8 @@ inline OutMap out_colmajor(int64_t M, int64_t N, int64_t ldc) { return OutMap{M,
 
 template <class T>
 void gemm_simt(cudaStream_t s, int64_t M, int64_t N, int64_t K, T alpha, const T* A, int64_t a_m,
-               int64_t a_k, const T* B, int64_t b_n, int64_t b_k, T beta, T* C, OutMap om);
+               int64_t a_k, const T* B, int64_t b_n, int64_t b_k, T beta, T* C, OutMap om,
+               const int* skip = nullptr);   // device flag: nothing is done when it is set
 
 // Tensor-core GEMM for K-major A [M][lda] and B [N][ldb] (k contiguous), every operand split
 // into two 11-bit halves: products that amortise it run on FP16 planes made beforehand (gemm_tc.cu),
@@ -192,9 +193,12 @@ void tri_inverse_upper_f64(cudaStream_t s, const double* R, int k, double* Rinv)
 void sym_eig_jacobi_f64(cudaStream_t s, double* G, int k, double* evec, double* eval, int* info);
 // One-sided Jacobi SVD of the k x k col-major Mat (destroyed): Mat = U diag(sigma) V^T,
 // sigma descending; U columns sorted, V columns in original order with order[rank] =
-// original column. ws_dev: >= 64 bytes of device scratch.
+// original column. ws_dev: >= svd_ws_bytes(k) of device scratch; work: svd_work_bytes(k), or null
+// (then FP64 sweeps alone).
+inline size_t svd_ws_bytes(int k) { return 256 + 8 * (size_t)k; }
+size_t svd_work_bytes(int k);
 void svd_jacobi_f64(cudaStream_t s, double* Mat, int k, double* U, double* sigma, double* V, int* order,
-                    int* info, void* ws_dev);
+                    int* info, void* ws_dev, void* work);
 
 void gather_cols_f64(cudaStream_t s, const double* V, const int* order, int k, double* out);
 

@@ -719,7 +719,7 @@ struct Engine : EngineBase {
     int* order = ar.get_n<int>(k);
     {
       Phase ph_(this, 2);
-      svd_jacobi_f64(s, Ms, k, Uj, sg, Vj, order, env->d_info, ar.get(64));
+      svd_jacobi_f64(s, Ms, k, Uj, sg, Vj, order, env->d_info, ar.get(svd_ws_bytes(k)), ar.get(svd_work_bytes(k)));
     }
     FP_CHECK(read_info() == 0, FPEPS_ERR_NUMERIC, "Jacobi SVD did not converge");
     r.U = Uj;
@@ -1297,7 +1297,7 @@ struct Engine : EngineBase {
       int* order = ar.get_n<int>(j);
       {
         Phase ph_(this, 2);
-        svd_jacobi_f64(s, Rm, j, Uj, sg, Vj, order, e->d_info, ar.get(64));
+        svd_jacobi_f64(s, Rm, j, Uj, sg, Vj, order, e->d_info, ar.get(svd_ws_bytes(j)), ar.get(svd_work_bytes(j)));
       }
       FP_CHECK(read_info() == 0, FPEPS_ERR_NUMERIC, "Jacobi SVD did not converge (fit)");
       double* Vs = ar.get_n<double>((int64_t)j * j);
@@ -1627,7 +1627,7 @@ struct Engine : EngineBase {
         int* order = ar.get_n<int>(rr);
         {
           Phase ph_(this, 2);
-          svd_jacobi_f64(s, Rm, rr, Uj, sg, Vj, order, e->d_info, ar.get(64));
+          svd_jacobi_f64(s, Rm, rr, Uj, sg, Vj, order, e->d_info, ar.get(svd_ws_bytes(rr)), ar.get(svd_work_bytes(rr)));
         }
         FP_CHECK(read_info() == 0, FPEPS_ERR_NUMERIC, "Jacobi SVD did not converge (sector fit)");
         double* Vs = ar.get_n<double>((int64_t)rr * rr);

@@ -94,7 +94,8 @@ template <class T, int BM, int BK>
 __global__ void __launch_bounds__(256) k_gemm(int64_t M, int64_t N, int64_t K, int64_t ks, T alpha,
                                               const T* __restrict__ A, int64_t a_m, int64_t a_k,
                                               const T* __restrict__ B, int64_t b_n, int64_t b_k, T beta,
-                                              T* __restrict__ C, OutMap om) {
+                                              T* __restrict__ C, OutMap om, const int* skip) {
+  if (skip && *skip) return;   // the same for every CTA of a cluster
   namespace cg = cooperative_groups;
   constexpr int TM = BM / 16;
   constexpr int TILE = BK * (BM + 1);
@@ -200,7 +201,8 @@ template <int BN, bool MF>
 __global__ void __launch_bounds__(256, 2) k_gemm_big(int64_t M, int64_t N, int64_t K, int64_t ks, float alpha,
                                                      const float* __restrict__ A, int64_t a_m, int64_t a_k,
                                                      const float* __restrict__ B, int64_t b_n, int64_t b_k, float beta,
-                                                     float* __restrict__ C, OutMap om) {
+                                                     float* __restrict__ C, OutMap om, const int* skip) {
+  if (skip && *skip) return;
   constexpr int TN = BN / 16;
   constexpr int ATILE = GK * GS, BTILE = GK * (BN + 2), HALF = GB / 2 * BN;
   __shared__ __align__(16) float sh[2 * (ATILE + BTILE) > HALF ? 2 * (ATILE + BTILE) : HALF];
@@ -346,33 +348,33 @@ void launch(void (*kern)(KArgs...), dim3 grid, cudaStream_t s, Args... args) {
 
 template <class T, int BM, int BK>
 void run_tile(cudaStream_t s, int split, int64_t M, int64_t N, int64_t K, T alpha, const T* A, int64_t a_m, int64_t a_k,
-              const T* B, int64_t b_n, int64_t b_k, T beta, T* C, OutMap om) {
+              const T* B, int64_t b_n, int64_t b_k, T beta, T* C, OutMap om, const int* skip) {
   const int64_t ks = ((K + BK - 1) / BK + split - 1) / split * BK;
   launch(k_gemm<T, BM, BK>, dim3((unsigned)((N + BM - 1) / BM), (unsigned)((M + BM - 1) / BM), (unsigned)split), s, M, N, K,
-         ks, alpha, A, a_m, a_k, B, b_n, b_k, beta, C, om);
+         ks, alpha, A, a_m, a_k, B, b_n, b_k, beta, C, om, skip);
 }
 
 template <int BN>
 void run_big(cudaStream_t s, int split, int64_t M, int64_t N, int64_t K, float alpha, const float* A, int64_t a_m,
-             int64_t a_k, const float* B, int64_t b_n, int64_t b_k, float beta, float* C, OutMap om) {
+             int64_t a_k, const float* B, int64_t b_n, int64_t b_k, float beta, float* C, OutMap om, const int* skip) {
   const int64_t ks = ((K + GK - 1) / GK + split - 1) / split * GK;
   launch(om.c1 == 1 ? k_gemm_big<BN, true> : k_gemm_big<BN, false>,
          dim3((unsigned)((N + BN - 1) / BN), (unsigned)((M + GB - 1) / GB), (unsigned)split), s, M, N, K, ks, alpha, A, a_m,
-         a_k, B, b_n, b_k, beta, C, om);
+         a_k, B, b_n, b_k, beta, C, om, skip);
 }
 
 }  // namespace
 
 template <class T>
 void gemm_simt(cudaStream_t s, int64_t M, int64_t N, int64_t K, T alpha, const T* A, int64_t a_m, int64_t a_k,
-               const T* B, int64_t b_n, int64_t b_k, T beta, T* C, OutMap om) {
+               const T* B, int64_t b_n, int64_t b_k, T beta, T* C, OutMap om, const int* skip) {
   if (M <= 0 || N <= 0) return;
   FP_CHECK(om.mdiv > 0 && om.ndiv > 0, FPEPS_ERR_ARG, "gemm: bad output map");
   FP_CHECK((M + 63) / 64 <= 65535, FPEPS_ERR_UNSUPPORTED, "gemm: M too large for grid");
   ProfToken pt = prof_begin(PROF_GEMM_SIMT, s, 2.0 * M * N * K,
                             (double)sizeof(T) * ((double)M * K + (double)N * K + (double)M * N));
   const Pick p = pick(M, N, K, sizeof(T) == 8, b_k == 1);
-  auto go = [&](auto run) { run(s, p.split, M, N, K, alpha, A, a_m, a_k, B, b_n, b_k, beta, C, om); };
+  auto go = [&](auto run) { run(s, p.split, M, N, K, alpha, A, a_m, a_k, B, b_n, b_k, beta, C, om, skip); };
   if (p.kind == 0) go(run_tile<T, 64, 16>);
   else if (p.kind == 1) go(run_tile<T, 32, 32>);
   else if (p.kind == 2) go(run_tile<T, 16, 64>);
@@ -386,8 +388,8 @@ void gemm_simt(cudaStream_t s, int64_t M, int64_t N, int64_t K, T alpha, const T
 }
 
 template void gemm_simt<float>(cudaStream_t, int64_t, int64_t, int64_t, float, const float*, int64_t, int64_t,
-                               const float*, int64_t, int64_t, float, float*, OutMap);
+                               const float*, int64_t, int64_t, float, float*, OutMap, const int*);
 template void gemm_simt<double>(cudaStream_t, int64_t, int64_t, int64_t, double, const double*, int64_t, int64_t,
-                                const double*, int64_t, int64_t, double, double*, OutMap);
+                                const double*, int64_t, int64_t, double, double*, OutMap, const int*);
 
 }  // namespace fpeps

@@ -1,19 +1,12 @@
 // Randomized-SVD building blocks (Sec. IV; Halko et al. 2011, Example 1.6):
-// the Gaussian sketch Omega, FP64 Gram matrices, Cholesky QR, the one-sided
-// Jacobi SVD of small matrices, norms and layout helpers.
+// the Gaussian sketch Omega, FP64 Gram matrices, Cholesky QR, norms and
+// layout helpers.
 //
 // Gaussian sketch: Philox4x64-10 (Salmon et al., SC'11) keyed by (seed, layer)
 // with counter (i >> 1, j, site | stage << 16, row | env << 16); the word pair
 // (x0,x1) for even i and (x2,x3) for odd i gives u = ((x >> 11) + 0.5) 2^-53
 // and z = sqrt(-2 ln u1) cos(2 pi u2) (Box-Muller). i is the flat row index of
 // the sketched space in C order of its (bond, bundle) legs.
-//
-// One-sided Jacobi SVD: Hestenes' method with the cyclic round-robin ordering;
-// each rotation makes two columns orthogonal (Demmel and Veselic 1992). The
-// path always applies it to the transposed triangular factor of a QR (the
-// preconditioned form of Drmac and Veselic 2008), where it converges in about
-// ten sweeps; the sweep count is capped at 30.
-#include <cstdio>
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -360,264 +353,6 @@ __global__ void __launch_bounds__(128) k_tri_inverse_warp(const double* R, int k
   for (int i = lane; i < k; i += 32) Rinv[(int64_t)i * k + j] = x[i];
 }
 
-// One round of the one-sided Jacobi method on the columns of M (col-major,
-// k x k) with the accumulated right rotations in V. Pairs of the round-robin
-// schedule: player positions 0..kk-1 (kk even), position 0 fixed.
-__device__ __forceinline__ int rr_player(int pos, int round, int kk) {
-  if (pos == 0) return 0;
-  return 1 + ((pos - 1 + round) % (kk - 1));
-}
-
-__global__ void __launch_bounds__(1024) k_jacobi_svd(double* M, double* V, int k, int max_sweeps, double eps,
-                                                      int* info) {
-  const int kk = (k % 2) ? k + 1 : k;   // dummy column k when odd
-  const int lane = threadIdx.x % 32, warp = threadIdx.x / 32, nwarp = blockDim.x / 32;
-  __shared__ int rotated;
-  __shared__ double fro2;
-  for (int e = threadIdx.x; e < k * k; e += blockDim.x) V[e] = ((e / k) == (e % k)) ? 1.0 : 0.0;
-  if (threadIdx.x == 0) {
-    double f = 0;
-    for (int64_t e = 0; e < (int64_t)k * k; ++e) f = fma(M[e], M[e], f);
-    fro2 = f;
-  }
-  __syncthreads();
-  // a column whose squared norm is below 1e-30 of the whole matrix carries no
-  // resolvable direction: rotations against it only stir rounding noise
-  const double tiny = 1e-30 * fro2;
-  int sweep = 0;
-  for (; sweep < max_sweeps; ++sweep) {
-    if (threadIdx.x == 0) rotated = 0;
-    __syncthreads();
-    for (int round = 0; round < kk - 1; ++round) {
-      for (int pr = warp; pr < kk / 2; pr += nwarp) {
-        int a = rr_player(pr, round, kk), b = rr_player(kk - 1 - pr, round, kk);
-        int p = min(a, b), q = max(a, b);
-        if (q >= k) continue;
-        double* mp = M + (int64_t)p * k;
-        double* mq = M + (int64_t)q * k;
-        double al = 0, be = 0, ga = 0;
-        for (int i = lane; i < k; i += 32) {
-          double x = mp[i], y = mq[i];
-          al = fma(x, x, al); be = fma(y, y, be); ga = fma(x, y, ga);
-        }
-        for (int o = 16; o; o >>= 1) {
-          al += __shfl_xor_sync(0xffffffffu, al, o);
-          be += __shfl_xor_sync(0xffffffffu, be, o);
-          ga += __shfl_xor_sync(0xffffffffu, ga, o);
-        }
-        if (ga == 0.0 || fmin(al, be) <= tiny || fabs(ga) <= eps * sqrt(al) * sqrt(be)) continue;
-        double zeta = (be - al) / (2.0 * ga);
-        double t = (zeta >= 0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-        double c = 1.0 / sqrt(1.0 + t * t), s = c * t;
-        for (int i = lane; i < k; i += 32) {
-          double x = mp[i], y = mq[i];
-          mp[i] = c * x - s * y;
-          mq[i] = s * x + c * y;
-          double vx = V[(int64_t)p * k + i], vy = V[(int64_t)q * k + i];
-          V[(int64_t)p * k + i] = c * vx - s * vy;
-          V[(int64_t)q * k + i] = s * vx + c * vy;
-        }
-        if (lane == 0) rotated = 1;
-      }
-      __syncthreads();
-    }
-    if (!rotated) break;
-    __syncthreads();
-  }
-  // reaching the sweep cap leaves the columns orthogonal to rounding level; it is not an error
-  if (threadIdx.x == 0) info[0] = 0;
-}
-
-// The same method spread over the whole GPU, in blocks of two columns (block b:
-// columns 2b and 2b + 1). A round-robin schedule over the blocks gives every CTA a
-// pair of blocks (A, B) per round; the CTA copies their four columns of M and of V to
-// shared memory and rotates the four cross pairs, two at a time ((a0,b0) (a1,b1), then
-// (a0,b1) (a1,b0)), after first rotating each block's own pair in the first round of a
-// sweep. Every column pair is visited once per sweep, as in the scalar cyclic order,
-// with one grid barrier per round of blocks. Each rotation is carried by two warps (one
-// half of the rows each, partial dot products exchanged in shared memory), so the four
-// warps of a CTA keep all four FP64 pipes of the SM busy: FP64 is the limit here (~2 FMA
-// per cycle per SM on this part; a rotation of two length-k columns of M and of V costs
-// ~11 k FMA).
-// ws[0..1]: sweep rotation counters (two, alternating), ws[2]: squared Frobenius norm,
-// ws[3]: sweeps used, ws[4..5]: counters of rotations above sqrt(big2) (alternating).
-constexpr int JB_THREADS = 128;
-
-// rotation of local columns (p, q) by the two warps h = 0, 1 of a pair slot: rows
-// [h * half, (h + 1) * half); part[6] holds the two halves' (alpha, beta, gamma)
-// *big (if given) is set when the rotation's |gamma| / sqrt(alpha beta) exceeds sqrt(big2)
-__device__ __forceinline__ bool jacobi_rotate_split(double* __restrict__ mp, double* __restrict__ mq,
-                                                    double* __restrict__ vp, double* __restrict__ vq, int k, int h,
-                                                    int lane, double* part, double eps, double tiny, bool* big,
-                                                    double big2) {
-  const int half = (k + 1) / 2, i0 = h * half, i1 = min(k, i0 + half);
-  double al = 0, be = 0, ga = 0;
-  for (int i = i0 + lane; i < i1; i += 32) {
-    const double x = mp[i], y = mq[i];
-    al = fma(x, x, al);
-    be = fma(y, y, be);
-    ga = fma(x, y, ga);
-  }
-  for (int o = 16; o; o >>= 1) {
-    al += __shfl_xor_sync(0xffffffffu, al, o);
-    be += __shfl_xor_sync(0xffffffffu, be, o);
-    ga += __shfl_xor_sync(0xffffffffu, ga, o);
-  }
-  if (lane == 0) {
-    part[3 * h + 0] = al;
-    part[3 * h + 1] = be;
-    part[3 * h + 2] = ga;
-  }
-  __syncthreads();
-  // both warps add the halves in the same order, so they take the same decision and angle
-  al = part[0] + part[3];
-  be = part[1] + part[4];
-  ga = part[2] + part[5];
-  // |gamma| <= eps sqrt(alpha beta) tested squared: FP64 sqrt and division are long serial
-  // latencies here (~680 and ~430 cycles), so the angle takes one of each plus one rsqrt:
-  // tan = sign(d) 2 gamma / (|d| + sqrt(d^2 + 4 gamma^2)), d = beta - alpha, which is
-  // sign(zeta) / (|zeta| + sqrt(1 + zeta^2)) with zeta = d / (2 gamma)
-  const bool rot = !(ga == 0.0 || fmin(al, be) <= tiny || ga * ga <= eps * eps * al * be);
-  if (rot) {
-    if (big && ga * ga > big2 * al * be) *big = true;
-    const double d = be - al, g2 = 2.0 * ga;
-    const double t = (d >= 0 ? g2 : -g2) / (fabs(d) + sqrt(fma(d, d, g2 * g2)));
-    const double c = rsqrt(fma(t, t, 1.0)), sn = c * t;
-    for (int i = i0 + lane; i < i1; i += 32) {
-      const double x = mp[i], y = mq[i], a = vp[i], b = vq[i];
-      mp[i] = c * x - sn * y;
-      mq[i] = sn * x + c * y;
-      vp[i] = c * a - sn * b;
-      vq[i] = sn * a + c * b;
-    }
-  }
-  return rot;
-}
-
-__global__ void __launch_bounds__(JB_THREADS) k_jacobi_svd_blk(double* M, double* V, int k, int max_sweeps,
-                                                                double eps, double big2, unsigned long long* ws) {
-  namespace cg = cooperative_groups;
-  cg::grid_group grid = cg::this_grid();
-  extern __shared__ double jsh[];   // M columns [4][k], V columns [4][k], partial dots [2][6]
-  double* sm = jsh;
-  double* sv = jsh + 4 * (int64_t)k;
-  double* part = jsh + 8 * (int64_t)k;
-  const int nb = (k + 1) / 2, nbe = nb + (nb & 1);   // blocks; a dummy block when nb is odd
-  const int lane = threadIdx.x % 32, warp = threadIdx.x / 32;
-  const int slot = warp / 2, h = warp % 2;           // pair slot and row half of this warp
-  double* fro2p = (double*)&ws[2];
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)k * k; e += (int64_t)gridDim.x * blockDim.x)
-    V[e] = ((e / k) == (e % k)) ? 1.0 : 0.0;
-  if (blockIdx.x == 0) {   // ||M||_F^2 by block 0
-    __shared__ double red[JB_THREADS / 32];
-    double f = 0;
-    for (int64_t e = threadIdx.x; e < (int64_t)k * k; e += blockDim.x) f = fma(M[e], M[e], f);
-    for (int o = 16; o; o >>= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
-    if (lane == 0) red[warp] = f;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double t = 0;
-      for (int w = 0; w < JB_THREADS / 32; ++w) t += red[w];
-      *fro2p = t;
-      ws[0] = ws[1] = ws[4] = ws[5] = 0;
-    }
-  }
-  grid.sync();
-  const double tiny = 1e-30 * (*fro2p);
-  // The rotation counter of sweep s lives in ws[s & 1] (its count of rotations above
-  // sqrt(big2) in ws[4 + (s & 1)]); every block reads it after the last
-  // round and a further barrier follows, so all blocks take the same break decision; the slot
-  // is cleared for sweep s+2 at round 1 of sweep s+1, after those reads.
-  for (int sweep = 0; sweep < max_sweeps; ++sweep) {
-    for (int round = 0; round < nbe - 1; ++round) {
-      if (round == 1 && blockIdx.x == 0 && threadIdx.x == 0) ws[(sweep + 1) & 1] = ws[4 + ((sweep + 1) & 1)] = 0;
-      const int A = rr_player((int)blockIdx.x, round, nbe), B = rr_player(nbe - 1 - (int)blockIdx.x, round, nbe);
-      // local columns 0, 1 (block A) and 2, 3 (block B); -1: absent
-      int col[4];
-      col[0] = 2 * A;
-      col[1] = 2 * A + 1;
-      col[2] = 2 * B;
-      col[3] = 2 * B + 1;
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (col[j] >= k) col[j] = -1;
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        for (int i = threadIdx.x; i < k; i += blockDim.x) {
-          const bool in = col[j] >= 0;
-          sm[j * k + i] = in ? M[(int64_t)col[j] * k + i] : 0.0;
-          sv[j * k + i] = in ? V[(int64_t)col[j] * k + i] : 0.0;
-        }
-      __syncthreads();
-      int nrot = 0;
-      bool big = false;
-      // inner rounds: the blocks' own pairs (first round of a sweep), then the cross pairs
-      // inner round 0: (0,1) (2,3); 1: (0,2) (1,3); 2: (0,3) (1,2) -- slot 0 takes the first pair
-      for (int ir = round == 0 ? 0 : 1; ir < 3; ++ir) {
-        const int p = ir == 0 ? 2 * slot : slot;
-        const int q = ir == 0 ? 2 * slot + 1 : (ir == 1 ? slot + 2 : 3 - slot);
-        double* pt = part + 6 * slot;
-        if (col[p] >= 0 && col[q] >= 0) {
-          if (jacobi_rotate_split(sm + p * k, sm + q * k, sv + p * k, sv + q * k, k, h, lane, pt, eps, tiny, &big,
-                                  big2))
-            ++nrot;
-        } else {
-          __syncthreads();   // the same barrier count as a rotating slot
-        }
-        __syncthreads();
-      }
-      if (h == 0 && lane == 0 && nrot) atomicAdd(&ws[sweep & 1], (unsigned long long)nrot);
-      if (h == 0 && lane == 0 && big) atomicAdd(&ws[4 + (sweep & 1)], 1ull);
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (col[j] >= 0)
-          for (int i = threadIdx.x; i < k; i += blockDim.x) {
-            M[(int64_t)col[j] * k + i] = sm[j * k + i];
-            V[(int64_t)col[j] * k + i] = sv[j * k + i];
-          }
-      grid.sync();
-    }
-    const unsigned long long rot = *(volatile unsigned long long*)&ws[sweep & 1];
-    const unsigned long long nbig = *(volatile unsigned long long*)&ws[4 + (sweep & 1)];
-    grid.sync();
-    if (blockIdx.x == 0 && threadIdx.x == 0) ws[3] = (unsigned long long)(sweep + 1);
-    // converged: no rotation, or only rotations below sqrt(big2) relative, after which the
-    // off-diagonal products are O(big2) = O(eps / k) (quadratic convergence), so the next
-    // sweep would find nothing above eps
-    if (rot == 0 || nbig == 0) break;
-  }
-}
-
-// sigma_j = |m_j|, U_j = m_j / sigma_j (0 when sigma_j == 0), written in
-// descending order of sigma (ties by index): sigma[rank], U[:, rank],
-// order[rank] = original column.
-__global__ void k_svd_finish(const double* M, int k, double* U, double* sigma, int* order) {
-  __shared__ double sig[1024];
-  __shared__ double fro2;
-  for (int j = threadIdx.x; j < k; j += blockDim.x) {
-    double s = 0;
-    for (int i = 0; i < k; ++i) s = fma(M[(int64_t)j * k + i], M[(int64_t)j * k + i], s);
-    sig[j] = sqrt(s);
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double f = 0;
-    for (int j = 0; j < k; ++j) f = fma(sig[j], sig[j], f);
-    fro2 = f;
-  }
-  __syncthreads();
-  // columns at or below the Jacobi negligibility level were never orthogonalised:
-  // they get a zero singular vector instead of a normalised rounding residue
-  for (int j = threadIdx.x; j < k; j += blockDim.x) {
-    int rank = 0;
-    for (int i = 0; i < k; ++i) rank += (sig[i] > sig[j]) || (sig[i] == sig[j] && i < j);
-    order[rank] = j;
-    sigma[rank] = sig[j];
-    double inv = (sig[j] > 0 && sig[j] * sig[j] > 1e-30 * fro2) ? 1.0 / sig[j] : 0.0;
-    for (int i = 0; i < k; ++i) U[(int64_t)rank * k + i] = M[(int64_t)j * k + i] * inv;
-  }
-}
-
 template <class T, class S>
 __global__ void k_convert(const S* in, T* out, int64_t n) {
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x)
@@ -909,55 +644,6 @@ void tri_inverse_upper_f64(cudaStream_t s, const double* R, int k, double* Rinv)
   }
   FP_CHECK(k <= 1024, FPEPS_ERR_UNSUPPORTED, "tri_inverse: k > 1024");
   k_tri_inverse_warp<<<(k + wpb - 1) / wpb, wpb * 32, smem, s>>>(R, k, Rinv);
-  FP_LAUNCH();
-}
-
-void svd_jacobi_f64(cudaStream_t s, double* Mat, int k, double* U, double* sigma, double* V, int* order, int* info,
-                    void* ws_dev) {
-  FP_CHECK(k <= 1024, FPEPS_ERR_UNSUPPORTED, "svd: k > 1024");
-  if (k <= 96) {
-    // stopping rule |m_p.m_q| <= sqrt(k) eps |m_p||m_q|: a dot product of length k
-    // carries rounding of that size, so a fixed 1e-15 could never be met
-    k_jacobi_svd<<<1, 1024, 0, s>>>(Mat, V, k, 30, 1e-15 * sqrt((double)k), info);
-    FP_LAUNCH();
-  } else {
-    // one CTA per pair of two-column blocks, all co-resident (cooperative launch)
-    const int nb = (k + 1) / 2, blocks = (nb + (nb & 1)) / 2;
-    const size_t smem = (8 * (size_t)k + 12) * sizeof(double);
-    static bool attr = false;
-    static int max_blocks = -1;
-    if (!attr) {
-      FP_CUDA(cudaFuncSetAttribute(k_jacobi_svd_blk, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)((8 * 1024 + 12) * sizeof(double))));
-      int dev = 0, sms = 0, per = 0;
-      FP_CUDA(cudaGetDevice(&dev));
-      FP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-      FP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_jacobi_svd_blk, JB_THREADS,
-                                                            (8 * 1024 + 12) * sizeof(double)));
-      max_blocks = sms * std::max(per, 0);
-      attr = true;
-    }
-    FP_CHECK(blocks <= max_blocks, FPEPS_ERR_CUDA, "svd: too few co-resident blocks");
-    void* fn = (void*)k_jacobi_svd_blk;
-    unsigned long long* ws = (unsigned long long*)ws_dev;
-    int max_sweeps = 30;
-    double eps = 1e-15 * sqrt((double)k);
-    double big2 = eps / k;
-    void* args[] = {&Mat, &V, &k, &max_sweeps, &eps, &big2, &ws};
-    ProfToken pt = prof_begin(PROF_FACTOR, s, 0.0, 16.0 * k * k);
-    count_launch();
-    FP_CUDA(cudaLaunchCooperativeKernel(fn, blocks, JB_THREADS, args, smem, s));
-    prof_end(pt, s);
-    FP_CUDA(cudaMemsetAsync(info, 0, sizeof(int), s));
-    static const bool trace = getenv("FPEPS_TRACE_SVD") != nullptr;   // diagnostics: sweeps used
-    if (trace) {
-      unsigned long long sw = 0;
-      FP_CUDA(cudaMemcpyAsync(&sw, ws + 3, sizeof(sw), cudaMemcpyDeviceToHost, s));
-      FP_CUDA(cudaStreamSynchronize(s));
-      fprintf(stderr, "[fpeps] jacobi k=%d sweeps=%llu\n", k, sw);
-    }
-  }
-  k_svd_finish<<<1, 1024, 0, s>>>(Mat, k, U, sigma, order);
   FP_LAUNCH();
 }
 

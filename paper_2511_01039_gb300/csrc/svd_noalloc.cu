@@ -1,5 +1,5 @@
 // Scratch-free variant of the small FP64 SVD (fpeps_svd_f64): the same
-// one-sided Jacobi kernels, with their working storage in a fixed device array
+// factorisation, with its working storage in a fixed device array
 // instead of memory obtained from cudaMallocAsync.
 //
 // Who needs it: callers that must not allocate device memory at the moment
@@ -9,9 +9,9 @@
 // an allocation could synchronise, fragment the pool or fail. They pass only
 // their input and output buffers; this entry point allocates nothing.
 //
-// The working storage is g_svd_scratch below: 2 k^2 doubles (working matrix and
-// accumulated rotations) + k ints (ordering) + 512 bytes of counters, for
-// k <= FPEPS_SVD_NOALLOC_MAX_K (256), about 1.05 MB. Every GPU that loads the
+// The working storage is g_svd_scratch below: 5 k^2 doubles (working matrix, accumulated
+// rotations and the refinement's products), k^2 floats (the FP32 sweeps), lists of rotations,
+// ordering, counters and norms, for k <= FPEPS_SVD_NOALLOC_MAX_K (256), about 3 MB. Every GPU that loads the
 // library holds it until the process exits. In host code the symbol names a
 // host-side stand-in, not device memory, so it is never handed to a kernel
 // directly: on the first call on a device (with that device current) its device
@@ -30,7 +30,9 @@ namespace fpeps {
 namespace {
 
 constexpr int kMaxK = FPEPS_SVD_NOALLOC_MAX_K;
-constexpr size_t kScratchBytes = 2 * (size_t)kMaxK * kMaxK * sizeof(double) + (size_t)kMaxK * sizeof(int) + 512;
+// two matrices, the factorisation's work (svd_work_bytes: three more, an FP32 copy and lists of rotations), order, counters and norms
+constexpr size_t kScratchBytes = 5 * (size_t)kMaxK * kMaxK * sizeof(double) + ((size_t)kMaxK + 1) * kMaxK * sizeof(float) + 70000 +
+                                 (size_t)kMaxK * (sizeof(int) + sizeof(double)) + 4096;
 static __device__ __align__(256) unsigned char g_svd_scratch[kScratchBytes];
 
 std::mutex g_mu;
@@ -65,13 +67,18 @@ extern "C" fpeps_status fpeps_svd_f64_noalloc(const double* M, int32_t k, double
     const size_t kk = (size_t)k * k;
     double* Mw = reinterpret_cast<double*>(scr);
     double* Vw = Mw + kk;
-    int* order = reinterpret_cast<int*>(Vw + kk);
-    char* ws = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(order + k) + 255) & ~uintptr_t(255));
-    int* info = reinterpret_cast<int*>(ws + 128);
-    // every region is rewritten before it is read: Mw by this copy, Vw, order and
-    // the counters by the Jacobi kernels (which reset their counters on entry)
+    char* work = reinterpret_cast<char*>(Vw + kk);   // 256-byte aligned regions from here on
+    auto up = [](size_t b) { return (b + 255) / 256 * 256; };
+    work = scr + up((size_t)(work - scr));
+    char* ws = work + up(fpeps::svd_work_bytes(k));
+    int* order = reinterpret_cast<int*>(ws + up(fpeps::svd_ws_bytes(k)));
+    int* info = reinterpret_cast<int*>(reinterpret_cast<char*>(order) + up((size_t)k * sizeof(int)));
+    if (reinterpret_cast<char*>(info) + sizeof(int) > scr + fpeps::kScratchBytes)
+      throw fpeps::Error{FPEPS_ERR_ARG, "svd scratch too small"};
+    // every region is rewritten before it is read: Mw by this copy, the rest by the
+    // factorisation (which clears its counters on entry)
     FP_CUDA(cudaMemcpyAsync(Mw, M, kk * sizeof(double), cudaMemcpyDeviceToDevice, s));
-    fpeps::svd_jacobi_f64(s, Mw, k, U, sigma, Vw, order, info, ws);
+    fpeps::svd_jacobi_f64(s, Mw, k, U, sigma, Vw, order, info, ws, work);
     fpeps::gather_cols_f64(s, Vw, order, k, V);
     FP_CUDA(cudaStreamSynchronize(s));
     return FPEPS_OK;
