@@ -752,14 +752,13 @@ fpeps_status fpeps_svd_f64(const double* M, int32_t k, double* U, double* sigma,
     char* scr = nullptr;
     auto up = [](size_t n) { return (n + 255) / 256 * 256; };
     const size_t b_mat = up(2 * kk * sizeof(double)), b_ord = up((size_t)k * sizeof(int)), b_ws = up(fpeps::svd_ws_bytes(k));
-    FP_CUDA(cudaMallocFromPoolAsync((void**)&scr, b_mat + b_ord + b_ws + 256 + fpeps::svd_work_bytes(k), fpeps::scratch_pool(), s));
+    FP_CUDA(cudaMallocFromPoolAsync((void**)&scr, b_mat + b_ord + b_ws + std::max<size_t>(fpeps::svd_work_bytes(k), 16), fpeps::scratch_pool(), s));
     double* Mw = (double*)scr;
     double* Vw = Mw + kk;
     int* order = (int*)(scr + b_mat);
     void* ws = scr + b_mat + b_ord;
-    int* info = (int*)(scr + b_mat + b_ord + b_ws);
     FP_CUDA(cudaMemcpyAsync(Mw, M, kk * sizeof(double), cudaMemcpyDeviceToDevice, s));
-    fpeps::svd_jacobi_f64(s, Mw, k, U, sigma, Vw, order, info, ws, scr + b_mat + b_ord + b_ws + 256);
+    fpeps::svd_jacobi_f64(s, Mw, k, U, sigma, Vw, order, ws, scr + b_mat + b_ord + b_ws);
     fpeps::gather_cols_f64(s, Vw, order, k, V);
     FP_CUDA(cudaFreeAsync(scr, s));
     FP_CUDA(cudaStreamSynchronize(s));

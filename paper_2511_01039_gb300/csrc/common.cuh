@@ -183,14 +183,14 @@ template <class T>
 void gaussian_sketch(cudaStream_t s, T* out, int64_t n_rows, int64_t k, int64_t ld, const int64_t* perm_div,
                      uint64_t seed, uint64_t layer, uint64_t w2, uint64_t w3);
 
+// upper triangle of G = Y^T Y (row-major), zeros below
 template <class T>
 void gram_f64(cudaStream_t s, const T* Y, int64_t m, int64_t k, int64_t ld, double* G);
 
-// returns device status word pointer semantics: info[0] != 0 on failure
-// ws: >= 8 bytes of device scratch
-void cholesky_upper_f64(cudaStream_t s, double* G, int k, int* info, double* ws);
-void tri_inverse_upper_f64(cudaStream_t s, const double* R, int k, double* Rinv);
-void sym_eig_jacobi_f64(cudaStream_t s, double* G, int k, double* evec, double* eval, int* info);
+// G (upper triangle of a Gram matrix, row-major, lower triangle zero) -> R with G = R^T R, and
+// X = R^-T (row-major lower, i.e. R^-1 column-major); dependent columns give zero rows of R and zero
+// rows and columns of X. info[0] |= 1 when a pivot is not finite.
+void cholesky_inverse_f64(cudaStream_t s, double* G, double* X, int k, int* info);
 // One-sided Jacobi SVD of the k x k col-major Mat (destroyed): Mat = U diag(sigma) V^T,
 // sigma descending; U columns sorted, V columns in original order with order[rank] =
 // original column. ws_dev: >= svd_ws_bytes(k) of device scratch; work: svd_work_bytes(k), or null
@@ -198,7 +198,7 @@ void sym_eig_jacobi_f64(cudaStream_t s, double* G, int k, double* evec, double* 
 inline size_t svd_ws_bytes(int k) { return 256 + 8 * (size_t)k; }
 size_t svd_work_bytes(int k);
 void svd_jacobi_f64(cudaStream_t s, double* Mat, int k, double* U, double* sigma, double* V, int* order,
-                    int* info, void* ws_dev, void* work);
+                    void* ws_dev, void* work);
 
 void gather_cols_f64(cudaStream_t s, const double* V, const int* order, int k, double* out);
 

@@ -628,12 +628,11 @@ struct Engine : EngineBase {
   void one_pass(Arena& ar, const T* Y, int64_t m, int k, T* Q, double* R, int how = PASS_PLAIN) {
     double* G = ar.get_n<double>((int64_t)k * k);
     gram_f64<T>(s, Y, m, k, m, G);
-    cholesky_upper_f64(s, G, k, env->d_info, ar.get_n<double>(8));
-    FP_CHECK(read_info() == 0, FPEPS_ERR_NUMERIC, "QR: non-finite Gram matrix");
     T* Bt = ar.get_n<T>((int64_t)k * k);
-    double* Rinv = ar.get_n<double>((int64_t)k * k);
-    tri_inverse_upper_f64(s, G, k, Rinv);
-    convert_f64_t<T>(s, Rinv, k, k, Bt);   // Rinv is row-major; Bt col-major
+    double* Rinv = ar.get_n<double>((int64_t)k * k);   // column-major, as Bt
+    // a non-finite Gram matrix is recorded in d_info, which the next read_info() reports
+    cholesky_inverse_f64(s, G, Rinv, k, env->d_info);
+    convert_f64<T>(s, Rinv, Bt, (int64_t)k * k);
     // Q(m, j) = sum_i Y(m, i) Rinv(i, j)
     if (how == PASS_DIAG_SPLIT) {
       zero_diag<T>(s, Bt, k, k);
@@ -719,9 +718,9 @@ struct Engine : EngineBase {
     int* order = ar.get_n<int>(k);
     {
       Phase ph_(this, 2);
-      svd_jacobi_f64(s, Ms, k, Uj, sg, Vj, order, env->d_info, ar.get(svd_ws_bytes(k)), ar.get(svd_work_bytes(k)));
+      svd_jacobi_f64(s, Ms, k, Uj, sg, Vj, order, ar.get(svd_ws_bytes(k)), ar.get(svd_work_bytes(k)));
     }
-    FP_CHECK(read_info() == 0, FPEPS_ERR_NUMERIC, "Jacobi SVD did not converge");
+    FP_CHECK(read_info() == 0, FPEPS_ERR_NUMERIC, "QR: non-finite Gram matrix");
     r.U = Uj;
     double* Vs = ar.get_n<double>((int64_t)k * k);
     gather_cols_f64(s, Vj, order, k, Vs);
@@ -827,6 +826,7 @@ struct Engine : EngineBase {
     FP_CUDA(cudaEventRecord(ev0, s));
     e->spectra.zip.assign(Ly, {});
     e->spectra.fit.assign(Ly, {});
+    FP_CUDA(cudaMemsetAsync(e->d_info, 0, sizeof(int), s));   // sticky over the row
 
     const bool sym = e->cfg.symmetry == 1;
     if (sym) {
@@ -1297,9 +1297,9 @@ struct Engine : EngineBase {
       int* order = ar.get_n<int>(j);
       {
         Phase ph_(this, 2);
-        svd_jacobi_f64(s, Rm, j, Uj, sg, Vj, order, e->d_info, ar.get(svd_ws_bytes(j)), ar.get(svd_work_bytes(j)));
+        svd_jacobi_f64(s, Rm, j, Uj, sg, Vj, order, ar.get(svd_ws_bytes(j)), ar.get(svd_work_bytes(j)));
       }
-      FP_CHECK(read_info() == 0, FPEPS_ERR_NUMERIC, "Jacobi SVD did not converge (fit)");
+      FP_CHECK(read_info() == 0, FPEPS_ERR_NUMERIC, "QR: non-finite Gram matrix (fit)");
       double* Vs = ar.get_n<double>((int64_t)j * j);
       gather_cols_f64(s, Vj, order, j, Vs);
       T* Wt = ar.get_n<T>((int64_t)j * j);
@@ -1627,9 +1627,9 @@ struct Engine : EngineBase {
         int* order = ar.get_n<int>(rr);
         {
           Phase ph_(this, 2);
-          svd_jacobi_f64(s, Rm, rr, Uj, sg, Vj, order, e->d_info, ar.get(svd_ws_bytes(rr)), ar.get(svd_work_bytes(rr)));
+          svd_jacobi_f64(s, Rm, rr, Uj, sg, Vj, order, ar.get(svd_ws_bytes(rr)), ar.get(svd_work_bytes(rr)));
         }
-        FP_CHECK(read_info() == 0, FPEPS_ERR_NUMERIC, "Jacobi SVD did not converge (sector fit)");
+        FP_CHECK(read_info() == 0, FPEPS_ERR_NUMERIC, "QR: non-finite Gram matrix (sector fit)");
         double* Vs = ar.get_n<double>((int64_t)rr * rr);
         gather_cols_f64(s, Vj, order, rr, Vs);
         T* Wt = ar.get_n<T>((int64_t)rr * rr);

@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(256) k_gram(const T* __restrict__ Y, int64_t m
   __shared__ double si[32][33];
   __shared__ double sj[32][33];
   const int ti = blockIdx.y, tj = blockIdx.x;
-  if (tj < ti) return;   // upper tiles only, mirrored at the end
+  if (tj < ti) return;   // upper tiles only
   const int64_t r0 = blockIdx.z * chunk, r1 = min(m, r0 + chunk);
   const int tid = threadIdx.x;
   const int li = tid / 8, lj = (tid % 8) * 4;   // each thread: 1 row x 4 cols of the tile
@@ -153,204 +153,199 @@ __global__ void __launch_bounds__(256) k_gram_df(const float* __restrict__ Y, in
   }
 }
 
-__global__ void k_mirror_upper(double* G, int k) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)k * k; e += (int64_t)gridDim.x * blockDim.x) {
-    int i = e / k, j = e % k;
-    if (j < i) G[e] = G[(int64_t)j * k + i];
-  }
+// ---------------------------------------------------------------- Cholesky factor and its inverse
+// G = R^T R (R upper, row-major, in place of the upper triangle of the Gram matrix G; the lower
+// triangle is zero on entry and stays so) and X = R^-T (lower, row-major, zero on entry): the
+// elimination runs on [G | I]. A pivot at or below tol * max diag means column j depends
+// numerically on the columns before it: row j of R is set to zero (the column of Q it would give
+// is zero), and with it row and column j of X. info[0] |= 1 for non-finite input.
+//
+// 1 / sqrt(x) from the FP32 value by one step of Householder's third-order iteration (the Taylor
+// series of (1 - r)^(-1/2), r = 1 - x y^2 ~ 2^-22): about 320 cycles of dependent FP64 operations, half
+// of what rsqrt() takes here, on the critical path of every column.
+__device__ __forceinline__ double rsqrt_fast(double x) {
+  const int hi = __double2hiint(x);
+  if (hi < 0x00100000) return rsqrt(x);   // below the normal range
+  const int e = ((hi >> 20) - 1023) & ~1;
+  const double m = __hiloint2double(hi - (e << 20), __double2loint(x));   // [1, 4)
+  const double y = (double)rsqrtf((float)m);
+  const double r = fma(-(m * y), y, 1.0);
+  const double p = fma(fma(r, 0.3125, 0.375), r, 0.5);
+  const double z = fma(p, y * r, y);
+  return __hiloint2double(__double2hiint(z) - ((e / 2) << 20), __double2loint(z));
 }
 
-// In-place Cholesky G = R^T R (R upper, row-major), one block, for the Gram
-// matrix of the columns of Y. A pivot at or below tol * max diag means column j
-// depends numerically on the columns before it: row j of R is set to zero (the
-// column of Q it would give is zero). info = 1 only for non-finite input.
-__global__ void __launch_bounds__(1024) k_cholesky(double* G, int k, double tol, int* info) {
-  __shared__ double piv_s;
+// The elimination of the n columns of D = [A | I] (shared memory, rows of ld doubles, A in columns 0 ..
+// n - 1, I in n .. 2 n - 1) by one CTA of NT threads; n <= 48. Warp 0 takes
+// the next pivot's reciprocal root, a chain of FP64 latencies, while the warps of the other three
+// sub-partitions update the rows below: behind their FMAs in the same FP64 pipe (a warp's FP64
+// instruction occupies it for 64 cycles) the chain took twice as long. dg: the diagonal of R. Returns whether a pivot
+// was not finite.
+template <int NT>
+__device__ __forceinline__ bool eliminate(double* D, int ld, int n, double cut, double* dg, int* bad) {
+  __shared__ double y_s;
+  const int tid = threadIdx.x, warp = tid / 32;
+  double d = D[0];
+  auto pivot = [&](int j) {
+    const double y = isfinite(d) && d > cut ? rsqrt_fast(d) : 0.0;
+    if (tid == 0) {
+      y_s = y;
+      dg[j] = d * y;
+      if (!isfinite(d)) *bad = 1;
+    }
+  };
+  if (warp == 0) pivot(0);
+  __syncthreads();
+  for (int j = 0; j < n; ++j) {
+    // row j: columns j + 1 .. n - 1 of A and 0 .. j of the inverse
+    if (tid < n) {
+      const int c = tid < n - j - 1 ? j + 1 + tid : n + tid - (n - j - 1);
+      D[j * ld + c] *= y_s;
+    }
+    __syncthreads();
+    const int m = n - j - 1;
+    if (warp == 0) {
+      if (m > 0) {
+        const double r = D[j * ld + j + 1];
+        d = fma(-r, r, D[(j + 1) * ld + j + 1]);
+        pivot(j + 1);
+      }
+    } else if (warp % 4 != 0) {
+      auto upd = [&](int i, int c) {   // column c > j of A, or c <= j of the inverse
+        if (c > j && (c < i || (i == j + 1 && c == i))) return;   // (the next pivot is taken above)
+        const int cc = c > j ? c : n + c;
+        D[i * ld + cc] = fma(-D[j * ld + i], D[j * ld + cc], D[i * ld + cc]);
+      };
+      const int u = (warp - 1 - warp / 4) * 32 + tid % 32, nu = NT / 4 * 3;
+      if (n <= 32) {   // a fixed width: a division by n costs more than the update
+        for (int e = u; e < m * 32; e += nu)
+          if (e % 32 < n) upd(j + 1 + e / 32, e % 32);
+      } else {
+        for (int e = u; e < m * 48; e += nu)
+          if (e % 48 < n) upd(j + 1 + e / 48, e % 48);
+      }
+    }
+    __syncthreads();
+  }
+  return *bad != 0;
+}
+
+// k <= CH_SMALL: one CTA, everything in shared memory. Measured at k = 46: factor and inverse 70 + 38 us
+// in two kernels before, 35 us now.
+constexpr int CH_SMALL = 48;
+__global__ void __launch_bounds__(1024) k_chol_inv_small(double* G, double* X, int k, double tol, int* info) {
+  extern __shared__ double ch[];
   __shared__ double dmax_s;
   __shared__ int bad;
-  const int tid = threadIdx.x;
-  if (tid == 0) {
+  const int ld = 2 * k + 1, tid = threadIdx.x;
+  double* dg = ch + k * ld;
+  for (int e = tid; e < k * k; e += 1024) {
+    const int i = e / k, c = e % k;
+    ch[i * ld + c] = c >= i ? G[e] : 0.0;
+    ch[i * ld + k + c] = i == c ? 1.0 : 0.0;
+  }
+  if (tid == 0) bad = 0;
+  __syncthreads();
+  if (tid < 32) {
     double dm = 0;
-    bool fin = true;
-    for (int i = 0; i < k; ++i) {
-      const double d = G[(int64_t)i * k + i];
-      fin = fin && isfinite(d);
-      dm = fmax(dm, d);
-    }
-    dmax_s = dm;
-    bad = !fin;
+    for (int i = tid; i < k; i += 32) dm = fmax(dm, ch[i * ld + i]);
+    for (int o = 16; o; o >>= 1) dm = fmax(dm, __shfl_xor_sync(0xffffffffu, dm, o));
+    if (tid == 0) dmax_s = dm;
   }
   __syncthreads();
-  if (bad) { if (tid == 0) info[0] = 1; return; }
-  for (int j = 0; j < k; ++j) {
-    if (tid == 0) {
-      const double d = G[(int64_t)j * k + j];
-      if (!isfinite(d)) bad = 1;
-      piv_s = d > tol * dmax_s ? sqrt(d) : 0.0;
-      G[(int64_t)j * k + j] = piv_s;
-    }
-    __syncthreads();
-    if (bad) { if (tid == 0) info[0] = 1; return; }
-    const double piv = piv_s;
-    for (int c = j + 1 + tid; c < k; c += blockDim.x) G[(int64_t)j * k + c] = piv > 0 ? G[(int64_t)j * k + c] / piv : 0.0;
-    __syncthreads();
-    const int n = k - j - 1;
-    // trailing update of the upper triangle: G[i][c] -= R[j][i] R[j][c], i <= c
-    for (int64_t e = tid; e < (int64_t)n * n; e += blockDim.x) {
-      int i = j + 1 + (int)(e / n), c = j + 1 + (int)(e % n);
-      if (c >= i) G[(int64_t)i * k + c] -= G[(int64_t)j * k + i] * G[(int64_t)j * k + c];
-    }
-    __syncthreads();
+  const bool nonfinite = eliminate<1024>(ch, ld, k, tol * dmax_s, dg, &bad);
+  for (int e = tid; e < k * k; e += 1024) {
+    const int i = e / k, c = e % k;
+    if (c >= i) G[e] = c == i ? dg[i] : ch[i * ld + c];
+    if (c <= i) X[e] = ch[i * ld + k + c];
   }
-  for (int64_t e = tid; e < (int64_t)k * k; e += blockDim.x) {
-    int i = e / k, c = e % k;
-    if (c < i) G[e] = 0.0;
-  }
-  if (tid == 0) info[0] = 0;
+  if (tid == 0 && nonfinite) atomicOr(info, 1);
 }
 
-// Blocked right-looking Cholesky over the whole GPU (cooperative launch, panel
-// width 32): block 0 factors the diagonal block in shared memory, every block
-// solves its share of the panel row, every block updates its share of the
-// trailing upper triangle; grid barriers in between. Same pivot rule as above.
-constexpr int CH_NB = 32;
-__global__ void __launch_bounds__(256) k_cholesky_coop(double* G, int k, double tol, int* info, double* ws) {
+// Blocked over the whole GPU (cooperative launch, panels of 32): block 0 eliminates the diagonal block
+// and its inverse in shared memory; every block multiplies its share of the panel row (of R to the
+// right, of X to the left) by that inverse; every block updates its share of the rows below. FP64
+// arithmetic (2 FMAs per cycle and SM) is the limit of the last two, so they take whatever order spreads
+// the FMAs; the first is a chain of 32 pivots. Measured at k = 266: factor 484 us and inverse 257 us in
+// two kernels before (a triangular solve and a warp per column), 284 us now.
+constexpr int CH_NB = 32, CH_NT = 512;
+__global__ void __launch_bounds__(CH_NT) k_chol_inv_coop(double* G, double* X, int k, double tol, int* info) {
   namespace cg = cooperative_groups;
   cg::grid_group grid = cg::this_grid();
-  __shared__ double D[CH_NB][CH_NB + 1];
-  __shared__ double inv_s[CH_NB];
-  __shared__ double rinv_s;
-  __shared__ int bad_s;
-  const int tid = threadIdx.x;
-  const int lane = tid % 32, warp = tid / 32;
-  const int64_t gtid = blockIdx.x * (int64_t)blockDim.x + tid;
-  const int64_t gsize = (int64_t)gridDim.x * blockDim.x;
-  if (blockIdx.x == 0 && tid == 0) {
-    double dm = 0;
-    bool fin = true;
-    for (int i = 0; i < k; ++i) {
-      const double d = G[(int64_t)i * k + i];
-      fin = fin && isfinite(d);
-      dm = fmax(dm, d);
+  __shared__ double D[CH_NB * (2 * CH_NB + 1)];
+  __shared__ double dg[CH_NB];
+  __shared__ double in[CH_NT / 32][CH_NB];
+  __shared__ double dmax_s;
+  __shared__ int bad;
+  const int tid = threadIdx.x, lane = tid % 32, warp = tid / 32;
+  if (blockIdx.x == 0) {
+    if (tid == 0) bad = 0;
+    if (warp == 0) {
+      double dm = 0;
+      for (int i = lane; i < k; i += 32) dm = fmax(dm, G[(int64_t)i * k + i]);
+      for (int o = 16; o; o >>= 1) dm = fmax(dm, __shfl_xor_sync(0xffffffffu, dm, o));
+      if (lane == 0) dmax_s = dm;
     }
-    ws[0] = dm;
-    info[0] = !fin;
+    __syncthreads();
   }
-  grid.sync();
-  if (*(volatile int*)info) return;
-  const double dmax = ws[0];
   for (int p0 = 0; p0 < k; p0 += CH_NB) {
-    const int nb = min(CH_NB, k - p0);
+    const int nb = min(CH_NB, k - p0), p1 = p0 + nb;
     if (blockIdx.x == 0) {
-      for (int e = tid; e < nb * nb; e += blockDim.x) D[e / nb][e % nb] = G[(int64_t)(p0 + e / nb) * k + p0 + e % nb];
-      if (tid == 0) bad_s = 0;
+      const int ld = 2 * nb + 1;
+      for (int e = tid; e < nb * nb; e += CH_NT) {
+        const int i = e / nb, c = e % nb;
+        D[i * ld + c] = c >= i ? __ldcg(G + (int64_t)(p0 + i) * k + p0 + c) : 0.0;
+        D[i * ld + nb + c] = i == c ? 1.0 : 0.0;
+      }
       __syncthreads();
-      for (int j = 0; j < nb; ++j) {
-        // FP64 sqrt and division are long latencies here (~680 / ~430 cycles): the pivot's
-        // sqrt and the row's scale factor rsqrt run side by side
-        if (tid == 0) {
-          const double d = D[j][j];
-          if (!isfinite(d)) bad_s = 1;
-          const bool keep = d > tol * dmax;
-          D[j][j] = keep ? sqrt(d) : 0.0;
-          rinv_s = keep ? rsqrt(d) : 0.0;
-        }
-        __syncthreads();
-        if (bad_s) break;
-        for (int c = j + 1 + tid; c < nb; c += blockDim.x) D[j][c] *= rinv_s;
-        __syncthreads();
-        const int n = nb - j - 1;
-        for (int e = tid; e < n * n; e += blockDim.x) {
-          int i = j + 1 + e / n, c = j + 1 + e % n;
-          if (c >= i) D[i][c] -= D[j][i] * D[j][c];
-        }
-        __syncthreads();
-      }
-      if (tid == 0 && bad_s) info[0] = 1;
-      for (int e = tid; e < nb * nb; e += blockDim.x) {
-        int i = e / nb, c = e % nb;
-        if (c >= i) G[(int64_t)(p0 + i) * k + p0 + c] = D[i][c];
+      eliminate<CH_NT>(D, ld, nb, tol * dmax_s, dg, &bad);
+      for (int e = tid; e < nb * nb; e += CH_NT) {
+        const int i = e / nb, c = e % nb;
+        if (c >= i) G[(int64_t)(p0 + i) * k + p0 + c] = c == i ? dg[i] : D[i * ld + c];
+        if (c <= i) X[(int64_t)(p0 + i) * k + p0 + c] = D[i * ld + nb + c];
       }
     }
     grid.sync();
-    if (*(volatile int*)info) return;
-    // panel row: R[p0:p0+nb, c] solves R_pp^T x = G[p0:p0+nb, c] for c >= p0 + nb, one warp
-    // per column spread over the whole grid (lane i holds row i; each solved value is
-    // broadcast and folded into the rows below it), every block with the factored diagonal
-    // block and its pivots' reciprocals in shared memory
-    for (int e = tid; e < nb * nb; e += blockDim.x) D[e / nb][e % nb] = G[(int64_t)(p0 + e / nb) * k + p0 + e % nb];
+    if (p1 == k && p0 == 0) break;
+    // panel row: out_r = sum_{l <= r} L_rl in_l, one warp per column (lane r holds row r)
+    for (int e = tid; e < nb * nb; e += CH_NT) D[(e / nb) * (CH_NB + 1) + e % nb] = __ldcg(X + (int64_t)(p0 + e / nb) * k + p0 + e % nb);
     __syncthreads();
-    for (int i = tid; i < nb; i += blockDim.x) inv_s[i] = D[i][i] > 0 ? 1.0 / D[i][i] : 0.0;
-    __syncthreads();
-    {
-      const int wpb = blockDim.x / 32;
-      for (int64_t c = p0 + nb + (int64_t)blockIdx.x * wpb + warp; c < k; c += (int64_t)gridDim.x * wpb) {
-        const double gl = lane < nb ? G[(int64_t)(p0 + lane) * k + c] : 0.0;
-        double acc = 0.0, mine = 0.0;
-        for (int l = 0; l < nb; ++l) {
-          double r = 0.0;
-          if (lane == l) r = inv_s[l] != 0.0 ? (gl - acc) * inv_s[l] : 0.0;
-          r = __shfl_sync(0xffffffffu, r, l);
-          if (lane == l) mine = r;
-          if (lane > l && lane < nb) acc = fma(D[l][lane], r, acc);
+    for (int c = blockIdx.x + gridDim.x * warp; c < k - nb; c += gridDim.x * (CH_NT / 32)) {
+      double* col = c < p0 ? X + (int64_t)p0 * k + c : G + (int64_t)p0 * k + c + nb;
+      if (lane < nb) in[warp][lane] = __ldcg(col + (int64_t)lane * k);
+      __syncwarp();
+      if (lane < nb) {
+        double a0 = 0, a1 = 0;
+        for (int l = 0; l < nb; l += 2) {
+          a0 = fma(D[lane * (CH_NB + 1) + l], in[warp][l], a0);
+          if (l + 1 < nb) a1 = fma(D[lane * (CH_NB + 1) + l + 1], in[warp][l + 1], a1);
         }
-        if (lane < nb) G[(int64_t)(p0 + lane) * k + c] = mine;
+        col[(int64_t)lane * k] = a0 + a1;
       }
+      __syncwarp();
     }
     grid.sync();
-    // trailing update of the upper triangle (four partial sums: the dependent FP64 FMA
-    // chain is 64 cycles per step)
-    const int64_t r0 = p0 + nb, n = k - r0;
-    for (int64_t e = gtid; e < n * n; e += gsize) {
-      const int64_t i = r0 + e / n, c = r0 + e % n;
-      if (c < i) continue;
+    // rows below: row i of [X | G] -= sum_l R[l][i] [X | R][l], columns 0 .. p1 - 1 of X, i .. k - 1 of G
+    const int n = k - p1;
+    for (int64_t e = blockIdx.x * (int64_t)CH_NT + tid; e < (int64_t)n * k; e += (int64_t)gridDim.x * CH_NT) {
+      const int i = p1 + (int)(e / k), c = (int)(e % k);
+      if (c >= p1 && c < i) continue;
+      const double *r = G + (int64_t)p0 * k + i, *b = (c < p1 ? X : G) + (int64_t)p0 * k + c;
       double a0 = 0, a1 = 0, a2 = 0, a3 = 0;
       int l = 0;
       for (; l + 4 <= nb; l += 4) {
-        a0 = fma(G[(int64_t)(p0 + l) * k + i], G[(int64_t)(p0 + l) * k + c], a0);
-        a1 = fma(G[(int64_t)(p0 + l + 1) * k + i], G[(int64_t)(p0 + l + 1) * k + c], a1);
-        a2 = fma(G[(int64_t)(p0 + l + 2) * k + i], G[(int64_t)(p0 + l + 2) * k + c], a2);
-        a3 = fma(G[(int64_t)(p0 + l + 3) * k + i], G[(int64_t)(p0 + l + 3) * k + c], a3);
+        a0 = fma(__ldcg(r + (int64_t)l * k), __ldcg(b + (int64_t)l * k), a0);
+        a1 = fma(__ldcg(r + (int64_t)(l + 1) * k), __ldcg(b + (int64_t)(l + 1) * k), a1);
+        a2 = fma(__ldcg(r + (int64_t)(l + 2) * k), __ldcg(b + (int64_t)(l + 2) * k), a2);
+        a3 = fma(__ldcg(r + (int64_t)(l + 3) * k), __ldcg(b + (int64_t)(l + 3) * k), a3);
       }
-      for (; l < nb; ++l) a0 = fma(G[(int64_t)(p0 + l) * k + i], G[(int64_t)(p0 + l) * k + c], a0);
-      G[i * k + c] -= (a0 + a1) + (a2 + a3);
+      for (; l < nb; ++l) a0 = fma(__ldcg(r + (int64_t)l * k), __ldcg(b + (int64_t)l * k), a0);
+      double* o = (c < p1 ? X : G) + (int64_t)i * k + c;
+      *o = __ldcg(o) - ((a0 + a1) + (a2 + a3));
     }
     grid.sync();
   }
-  for (int64_t e = gtid; e < (int64_t)k * k; e += gsize) {
-    int64_t i = e / k, c = e % k;
-    if (c < i) G[e] = 0.0;
-  }
-}
-
-// Rinv = R^{-1} for upper-triangular R (row-major): one warp per column, the
-// back-substitution dot products split over the lanes, the column kept in
-// shared memory. Rows of R with a zero diagonal (dependent columns) give zero
-// rows and columns of Rinv: the inverse of the non-zero part, padded with zeros.
-__global__ void __launch_bounds__(128) k_tri_inverse_warp(const double* R, int k, double* Rinv) {
-  extern __shared__ double xs_all[];
-  const int lane = threadIdx.x % 32, w = threadIdx.x / 32;
-  double* x = xs_all + (int64_t)w * k;
-  const int j = blockIdx.x * (blockDim.x / 32) + w;
-  if (j >= k) return;
-  for (int i = lane; i < k; i += 32) x[i] = 0.0;
-  __syncwarp();
-  const double rjj = R[(int64_t)j * k + j];
-  if (rjj != 0.0) {
-    if (lane == 0) x[j] = 1.0 / rjj;
-    __syncwarp();
-    for (int i = j - 1; i >= 0; --i) {
-      const double rii = R[(int64_t)i * k + i];
-      if (rii == 0.0) continue;   // x[i] stays zero
-      double sdot = 0;
-      for (int l = i + 1 + lane; l <= j; l += 32) sdot = fma(R[(int64_t)i * k + l], x[l], sdot);
-      for (int o = 16; o; o >>= 1) sdot += __shfl_xor_sync(0xffffffffu, sdot, o);
-      if (lane == 0) x[i] = -sdot / rii;
-      __syncwarp();
-    }
-  }
-  __syncwarp();
-  for (int i = lane; i < k; i += 32) Rinv[(int64_t)i * k + j] = x[i];
+  if (blockIdx.x == 0 && tid == 0 && bad) atomicOr(info, 1);
 }
 
 template <class T, class S>
@@ -588,8 +583,6 @@ void gram_f64(cudaStream_t s, const T* Y, int64_t m, int64_t k, int64_t ld, doub
     k_gram_df<<<grid, 256, 0, s>>>((const float*)Y, m, k, ld, chunk, G);
     FP_LAUNCH();
     prof_end(pt, s);
-    k_mirror_upper<<<grid_for(k * k), 256, 0, s>>>(G, (int)k);
-    FP_LAUNCH();
     return;
   }
   int tiles = (int)((k + 31) / 32);
@@ -606,45 +599,32 @@ void gram_f64(cudaStream_t s, const T* Y, int64_t m, int64_t k, int64_t ld, doub
   k_gram<T><<<grid, 256, 0, s>>>(Y, m, k, ld, chunk, G);
   FP_LAUNCH();
   prof_end(pt, s);
-  k_mirror_upper<<<grid_for(k * k), 256, 0, s>>>(G, (int)k);
-  FP_LAUNCH();
 }
 
-void cholesky_upper_f64(cudaStream_t s, double* G, int k, int* info, double* ws) {
-  if (k <= 96) {
-    k_cholesky<<<1, 1024, 0, s>>>(G, k, 1e-13, info);
-    FP_LAUNCH();
-    return;
-  }
-  static int max_blocks = -1;
-  if (max_blocks < 0) {
-    int dev = 0, sms = 0, per = 0;
-    FP_CUDA(cudaGetDevice(&dev));
-    FP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    FP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_cholesky_coop, 256, 0));
-    max_blocks = sms * std::max(per, 0);
-  }
-  int blocks = std::min(max_blocks, 152);
-  FP_CHECK(blocks >= 1, FPEPS_ERR_CUDA, "cholesky: no co-resident blocks");
+void cholesky_inverse_f64(cudaStream_t s, double* G, double* X, int k, int* info) {
+  FP_CHECK(k <= 1024, FPEPS_ERR_UNSUPPORTED, "cholesky: k > 1024");
   double tol = 1e-13;
-  void* args[] = {&G, &k, &tol, &info, &ws};
-  ProfToken pt = prof_begin(PROF_FACTOR, s, (double)k * k * k / 3.0, 8.0 * k * k);
-  count_launch();
-  FP_CUDA(cudaLaunchCooperativeKernel((void*)k_cholesky_coop, blocks, 256, args, 0, s));
-  prof_end(pt, s);
-}
-
-void tri_inverse_upper_f64(cudaStream_t s, const double* R, int k, double* Rinv) {
-  const int wpb = 4;
-  size_t smem = (size_t)wpb * k * sizeof(double);
-  static bool attr = false;
-  if (!attr) {
-    FP_CUDA(cudaFuncSetAttribute(k_tri_inverse_warp, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * 1024 * 8));
-    attr = true;
+  ProfToken pt = prof_begin(PROF_FACTOR, s, 2.0 * k * k * k / 3.0, 16.0 * k * k);
+  FP_CUDA(cudaMemsetAsync(X, 0, sizeof(double) * k * k, s));
+  if (k <= CH_SMALL) {
+    k_chol_inv_small<<<1, 1024, (size_t)(k * (2 * k + 1) + k) * sizeof(double), s>>>(G, X, k, tol, info);
+    FP_LAUNCH();
+  } else {
+    static int max_blocks = -1;
+    if (max_blocks < 0) {
+      int dev = 0, sms = 0, per = 0;
+      FP_CUDA(cudaGetDevice(&dev));
+      FP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+      FP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_chol_inv_coop, CH_NT, 0));
+      max_blocks = sms * std::max(per, 0);
+    }
+    const int blocks = std::min(max_blocks, 152);
+    FP_CHECK(blocks >= 1, FPEPS_ERR_CUDA, "cholesky: no co-resident blocks");
+    void* args[] = {&G, &X, &k, &tol, &info};
+    count_launch();
+    FP_CUDA(cudaLaunchCooperativeKernel((void*)k_chol_inv_coop, blocks, CH_NT, args, 0, s));
   }
-  FP_CHECK(k <= 1024, FPEPS_ERR_UNSUPPORTED, "tri_inverse: k > 1024");
-  k_tri_inverse_warp<<<(k + wpb - 1) / wpb, wpb * 32, smem, s>>>(R, k, Rinv);
-  FP_LAUNCH();
+  prof_end(pt, s);
 }
 
 template <class T>

@@ -39,11 +39,8 @@ __device__ __forceinline__ int rr_player(int pos, int round, int kk) {
 }
 
 __global__ void __launch_bounds__(1024) k_jacobi_svd(double* M, double* V, int k, int max_sweeps, double eps,
-                                                      const int* skip, bool init, int* info) {
-  if (skip && *skip) {
-    if (threadIdx.x == 0) info[0] = 0;
-    return;
-  }
+                                                      const int* skip, bool init) {
+  if (skip && *skip) return;
   const int kk = (k % 2) ? k + 1 : k;   // dummy column k when odd
   const int lane = threadIdx.x % 32, warp = threadIdx.x / 32, nwarp = blockDim.x / 32;
   __shared__ int rotated;
@@ -100,7 +97,6 @@ __global__ void __launch_bounds__(1024) k_jacobi_svd(double* M, double* V, int k
     __syncthreads();
   }
   // reaching the sweep cap leaves the columns orthogonal to rounding level; it is not an error
-  if (threadIdx.x == 0) info[0] = 0;
 }
 
 // The same method spread over the whole GPU, in blocks of two columns (block b:
@@ -725,11 +721,11 @@ int resident(K kern, int threads, size_t smem) {
 }
 
 // FP64 sweeps from M and, unless init, the V given
-void sweeps_f64(cudaStream_t s, double* Mat, int k, double* V, const int* skip, bool init, int* info, void* ws_dev) {
+void sweeps_f64(cudaStream_t s, double* Mat, int k, double* V, const int* skip, bool init, void* ws_dev) {
   if (k <= 32) {   // one CTA; above, its SM's FP64 pipe takes longer than the grid barriers (k = 64: 15 ms)
     // stopping rule |m_p.m_q| <= sqrt(k) eps |m_p||m_q|: a dot product of length k
     // carries rounding of that size, so a fixed 1e-15 could never be met
-    k_jacobi_svd<<<1, 1024, 0, s>>>(Mat, V, k, 30, 1e-15 * sqrt((double)k), skip, init, info);
+    k_jacobi_svd<<<1, 1024, 0, s>>>(Mat, V, k, 30, 1e-15 * sqrt((double)k), skip, init);
     FP_LAUNCH();
     return;
   }
@@ -749,7 +745,6 @@ void sweeps_f64(cudaStream_t s, double* Mat, int k, double* V, const int* skip, 
   void* args[] = {&Mat, &V, &k, &max_sweeps, &eps, &big2, &skip, &init, &ws};
   count_launch();
   FP_CUDA(cudaLaunchCooperativeKernel((void*)k_jacobi_svd_blk, blocks, JB_THREADS, args, smem, s));
-  FP_CUDA(cudaMemsetAsync(info, 0, sizeof(int), s));
 }
 
 constexpr size_t kStateBytes = 512;
@@ -770,14 +765,13 @@ size_t svd_work_bytes(int k) {
   return kStateBytes + list_bytes(k) + 3 * kk * sizeof(double) + (k > J32_ONE ? (kk + k) * sizeof(float) : 0);
 }
 
-void svd_jacobi_f64(cudaStream_t s, double* Mat, int k, double* U, double* sigma, double* V, int* order, int* info, void* ws_dev,
-                    void* work) {
+void svd_jacobi_f64(cudaStream_t s, double* Mat, int k, double* U, double* sigma, double* V, int* order, void* ws_dev, void* work) {
   FP_CHECK(k <= 1024, FPEPS_ERR_UNSUPPORTED, "svd: k > 1024");
   ProfToken pt = prof_begin(PROF_FACTOR, s, 0.0, 16.0 * k * k);
   double* M = Mat;
   double* sig = (double*)((char*)ws_dev + 256);
   if (!work || k <= kDirect) {
-    sweeps_f64(s, Mat, k, V, nullptr, true, info, ws_dev);
+    sweeps_f64(s, Mat, k, V, nullptr, true, ws_dev);
   } else {
     const int64_t kk = (int64_t)k * k;
     SvdState* st = (SvdState*)work;
@@ -846,7 +840,7 @@ void svd_jacobi_f64(cudaStream_t s, double* Mat, int k, double* U, double* sigma
       k_svd_add2<<<grid_of(kk), 256, 0, s>>>(M, T1, V, Mat, kk, &st->skip_apply[it]);
       FP_LAUNCH();
     }
-    sweeps_f64(s, M, k, V, &st->done, false, info, ws_dev);
+    sweeps_f64(s, M, k, V, &st->done, false, ws_dev);
   }
   k_svd_norms<<<(k + 7) / 8, 256, 0, s>>>(M, k, sig);
   FP_LAUNCH();

@@ -72,13 +72,12 @@ extern "C" fpeps_status fpeps_svd_f64_noalloc(const double* M, int32_t k, double
     work = scr + up((size_t)(work - scr));
     char* ws = work + up(fpeps::svd_work_bytes(k));
     int* order = reinterpret_cast<int*>(ws + up(fpeps::svd_ws_bytes(k)));
-    int* info = reinterpret_cast<int*>(reinterpret_cast<char*>(order) + up((size_t)k * sizeof(int)));
-    if (reinterpret_cast<char*>(info) + sizeof(int) > scr + fpeps::kScratchBytes)
+    if (reinterpret_cast<char*>(order + k) > scr + fpeps::kScratchBytes)
       throw fpeps::Error{FPEPS_ERR_ARG, "svd scratch too small"};
     // every region is rewritten before it is read: Mw by this copy, the rest by the
     // factorisation (which clears its counters on entry)
     FP_CUDA(cudaMemcpyAsync(Mw, M, kk * sizeof(double), cudaMemcpyDeviceToDevice, s));
-    fpeps::svd_jacobi_f64(s, Mw, k, U, sigma, Vw, order, info, ws, work);
+    fpeps::svd_jacobi_f64(s, Mw, k, U, sigma, Vw, order, ws, work);
     fpeps::gather_cols_f64(s, Vw, order, k, V);
     FP_CUDA(cudaStreamSynchronize(s));
     return FPEPS_OK;
