@@ -266,7 +266,7 @@ __global__ void __launch_bounds__(P_THREADS, 1) k_gemm_tf32x3_t(const __grid_con
           if (handoff_abort(false)) { ok = false; break; }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const int st = it % T_STAGES, as = PAIR ? it % NSLOT : st;
-          if (lane == 0) {
+          if (elect_one()) {
             const uint32_t ah = tmem + abase + (uint32_t)(as * AW), al = ah + AW / 2;
             const uint64_t bh = sdesc(B_hi(st)), bl = sdesc(B_lo(st));
 #pragma unroll
@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(P_THREADS, 1) k_gemm_tf32x3_t(const __grid_con
         }
       }
     }
-    if (lane == 0) {
+    if (elect_one()) {
       mma_commit<PAIR>(drain, 1);
       const unsigned long long t0 = clock64();
       while (!mbar_try_wait(drain, 0) && clock64() - t0 < WAIT_LIMIT) {

@@ -27,7 +27,10 @@
 // epilogue (adds the D2 halves; releases D2 before its stores), 12-15 transposer. A tcgen05.mma
 // occupies its issuing thread for roughly the same ~100 cycles at any N up to ~200 (measured on
 // GB300, M = 128, kind::tf32), so the narrow bra products are issued from two threads, and the ket
-// of the next pair, issued from a third, overlaps the bra of the current one. Every wait is
+// of the next pair, issued from a third, overlaps the bra of the current one. The issuing warps run
+// their loops whole, with the MMAs under an elected lane; with all of it under lane 0 every MMA took
+// longer to issue (an interior site of the 8x8, chi = 500 size, k = 46: 4.13 -> 3.95 ms; of the 6x6,
+// chi = 256 size, k = 266: 6.25 -> 5.76 ms). Every wait is
 // bounded; on a timeout the CTA raises its abort flag, waits (bounded) for its bulk copies and
 // MMAs, frees its tensor memory and exits.
 #include <algorithm>
@@ -254,7 +257,8 @@ __global__ void __launch_bounds__(SW_THREADS, 1) k_sandwich_tc(const SwArgs a) {
     }
   } else if (warp == W_MMA) {
     // ket MMAs: the channels of pair k into D1, once the transposer has read pair k - 1
-    if (lane == 0) {
+    {
+      const bool leader = elect_one();
       const uint32_t idesc1 = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(a.n1p >> 3) << 17) | ((128u >> 4) << 24);
       const uint32_t lbo1 = (uint32_t)(a.n1p / 8) * 128;
       PairIter kp;
@@ -276,18 +280,22 @@ __global__ void __launch_bounds__(SW_THREADS, 1) k_sandwich_tc(const SwArgs a) {
 #pragma unroll
           for (int kk = 0; kk < KPAD / 8; ++kk) {
             const uint32_t acc = (c > kp.c0() || kk > 0) ? 1u : 0u;
-            mma_ts(tmem + TM_D1, al + kk * 8, sdesc_noswz(bh + 2 * kk * lbo1, lbo1, 128), idesc1, acc);
-            mma_ts(tmem + TM_D1, ah + kk * 8, sdesc_noswz(bl + 2 * kk * lbo1, lbo1, 128), idesc1, 1u);
-            mma_ts(tmem + TM_D1, ah + kk * 8, sdesc_noswz(bh + 2 * kk * lbo1, lbo1, 128), idesc1, 1u);
+            if (leader) {
+              mma_ts(tmem + TM_D1, al + kk * 8, sdesc_noswz(bh + 2 * kk * lbo1, lbo1, 128), idesc1, acc);
+              mma_ts(tmem + TM_D1, ah + kk * 8, sdesc_noswz(bl + 2 * kk * lbo1, lbo1, 128), idesc1, 1u);
+              mma_ts(tmem + TM_D1, ah + kk * 8, sdesc_noswz(bh + 2 * kk * lbo1, lbo1, 128), idesc1, 1u);
+            }
           }
-          mma_commit<false>(&kb_empty[st]);
-          mma_commit<false>(ka_empty);
+          if (leader) {
+            mma_commit<false>(&kb_empty[st]);
+            mma_commit<false>(ka_empty);
+          }
         }
         if (!ok) break;
-        mma_commit<false>(d1_full);
+        if (leader) mma_commit<false>(d1_full);
         ++k;
       }
-      drain_mmas(drain);
+      if (leader) drain_mmas(drain);
     }
     __syncwarp();
   } else if (warp == W_BRA0 || warp == W_BRA0 + 1) {
@@ -296,7 +304,8 @@ __global__ void __launch_bounds__(SW_THREADS, 1) k_sandwich_tc(const SwArgs a) {
     // accumulates them into D2 half w; the epilogue adds the halves. A tcgen05.mma costs its
     // issuing thread about the same time for any N up to ~200, so two issuers run the narrow
     // (N = 48) bra products at twice the rate of one.
-    if (lane == 0) {
+    {
+      const bool leader = elect_one();
       const int w = warp - W_BRA0;
       const uint32_t idesc2 = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(a.n2p >> 3) << 17) | ((128u >> 4) << 24);
       const uint32_t lbo2 = (uint32_t)(a.n2p / 8) * 128;
@@ -322,18 +331,20 @@ __global__ void __launch_bounds__(SW_THREADS, 1) k_sandwich_tc(const SwArgs a) {
           const uint8_t* bl = bh + ar_bytes;
           for (int kk = 0; kk < nkk2; ++kk) {
             const uint32_t acc = (!first || kk > 0) ? 1u : 0u;
-            mma_ts(d, al + kk * 8, sdesc_noswz(bh + 2 * kk * lbo2, lbo2, 128), idesc2, acc);
-            mma_ts(d, ah + kk * 8, sdesc_noswz(bl + 2 * kk * lbo2, lbo2, 128), idesc2, 1u);
-            mma_ts(d, ah + kk * 8, sdesc_noswz(bh + 2 * kk * lbo2, lbo2, 128), idesc2, 1u);
+            if (leader) {
+              mma_ts(d, al + kk * 8, sdesc_noswz(bh + 2 * kk * lbo2, lbo2, 128), idesc2, acc);
+              mma_ts(d, ah + kk * 8, sdesc_noswz(bl + 2 * kk * lbo2, lbo2, 128), idesc2, 1u);
+              mma_ts(d, ah + kk * 8, sdesc_noswz(bh + 2 * kk * lbo2, lbo2, 128), idesc2, 1u);
+            }
           }
-          mma_commit<false>(&ba_empty[w]);
+          if (leader) mma_commit<false>(&ba_empty[w]);
           first = false;
         }
         if (!ok) break;
-        mma_commit<false>(d2_full);
+        if (leader) mma_commit<false>(d2_full);
         ++b;
       }
-      drain_mmas(drain);
+      if (leader) drain_mmas(drain);
     }
     __syncwarp();
   } else if (warp >= W_KA0 && warp < W_EP0) {
