@@ -326,8 +326,8 @@ fpeps_status fpeps_apply_theta_op(fpeps_env* env, int32_t op, int32_t c, int32_t
 
 /* One contraction GEMM of the path on caller device buffers (diagnostic):
  * C[M][N] (row-major) = sum_k A[m][k] B[n][k]; A [M][lda], B [N][ldb] fp32.
- * mode FPEPS_F32: CUDA-core FP32; FPEPS_TF32X3 / FPEPS_BF16X3: tensor-core
- * 3xTF32 / 3xBF16 (needs K >= 32, lda and ldb multiples of 4, 16-byte aligned
+ * mode FPEPS_F32: CUDA-core FP32; FPEPS_TF32X3 / FPEPS_BF16X3: 22-bit split
+ * products on the tensor cores (needs K >= 32, lda and ldb multiples of 4, 16-byte aligned
  * A and B, else FPEPS_ERR_UNSUPPORTED). Synchronises `cuda_stream` for the
  * tensor-core modes. */
 fpeps_status fpeps_gemm_f32(int32_t mode, int64_t M, int64_t N, int64_t K, const float* A, int64_t lda,
