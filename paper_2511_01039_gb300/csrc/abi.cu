@@ -44,6 +44,22 @@ static cudaMemPool_t scratch_pool() {
   return pool;
 }
 
+// Pinned word for the status that a call without a handle reads back, one per thread: into pageable
+// memory the copy goes through the driver's staging (1000 x 2000 x 500: 46.0 -> 43.5 us a call). Null if it can't be had: a word on the
+// stack serves then.
+struct StatusWord {
+  int* p = nullptr;
+  StatusWord() {
+    if (cudaHostAlloc((void**)&p, sizeof(int), cudaHostAllocPortable) != cudaSuccess) {
+      cudaGetLastError();
+      p = nullptr;
+    }
+  }
+  ~StatusWord() {
+    if (p) cudaFreeHost(p);
+  }
+};
+
 static void trim_pools() {
   std::lock_guard<std::mutex> lk(g_pool_mu);
   for (auto& p : g_pools) cudaMemPoolTrimTo(p.second, 0);
@@ -736,11 +752,13 @@ fpeps_status fpeps_gemm_f32(int32_t mode, int64_t M, int64_t N, int64_t K, const
     FP_CUDA(cudaMallocFromPoolAsync((void**)&err, sb, fpeps::scratch_pool(), s));
     FP_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
     fpeps::gemm_tc(s, M, N, K, A, lda, B, ldb, C, om, err, sb);
-    int h = 0;
-    FP_CUDA(cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, s));
+    static thread_local fpeps::StatusWord word;
+    int on_stack = 0;
+    int* const h = word.p ? word.p : &on_stack;
+    FP_CUDA(cudaMemcpyAsync(h, err, sizeof(int), cudaMemcpyDeviceToHost, s));
     FP_CUDA(cudaStreamSynchronize(s));
     cudaFreeAsync(err, s);
-    if (h) throw Error{FPEPS_ERR_TIMEOUT, "tensor-core GEMM timed out"};
+    if (*h) throw Error{FPEPS_ERR_TIMEOUT, "tensor-core GEMM timed out"};
   });
 }
 
