@@ -340,7 +340,8 @@ fpeps_status fpeps_gemm_f32(int32_t mode, int64_t M, int64_t N, int64_t K, const
  * The path passes the transposed triangular factor of a QR, for which the
  * method converges in about ten sweeps (most of them in FP32, then corrected and
  * checked in FP64); the sweep count is capped at 30, so a badly conditioned
- * general matrix may return before full convergence.
+ * general matrix may return before full convergence. A NaN or an infinity in M
+ * comes back as NaN or infinite singular values.
  * Takes its scratch (about 5.5 k^2 doubles) stream-ordered on `cuda_stream` from a
  * pool of the library, and synchronises the stream. */
 fpeps_status fpeps_svd_f64(const double* M, int32_t k, double* U, double* sigma, double* V, void* cuda_stream);

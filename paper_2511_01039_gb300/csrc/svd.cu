@@ -674,17 +674,22 @@ __global__ void __launch_bounds__(256) k_svd_norms(const double* M, int k, doubl
 }
 
 // U_j = m_j / sigma_j (0 when sigma_j is negligible), written in descending order of sigma (ties by
-// index): sigma[rank], U[:, rank], order[rank] = original column. One block per column.
+// index): sigma[rank], U[:, rank], order[rank] = original column. One block per column. The ranks are
+// those of the bit patterns, a total order (NaN above infinity), so that order is a permutation whatever
+// the input: its entries index V (gather_cols_f64).
+__device__ __forceinline__ unsigned long long order_key(double s) { return (unsigned long long)__double_as_longlong(fabs(s)); }
 __global__ void __launch_bounds__(128) k_svd_emit(const double* M, const double* sig, int k, double* U, double* sigma, int* order) {
   const int j = blockIdx.x;
   const double sj = sig[j];
+  const unsigned long long kj = order_key(sj);
   __shared__ int rk[4];
   __shared__ double fr[4];
   int r = 0;
   double f = 0;
   for (int i = threadIdx.x; i < k; i += 128) {
     const double s = sig[i];
-    r += (s > sj) || (s == sj && i < j);
+    const unsigned long long ki = order_key(s);
+    r += ki > kj || (ki == kj && i < j);
     f = fma(s, s, f);
   }
   for (int o = 16; o; o >>= 1) {
