@@ -296,13 +296,13 @@ __global__ void __launch_bounds__(P_THREADS, 1) k_gemm_f16x3(const __grid_consta
       while (ok && wi.next(g, w)) {
         for (int c = w.c0; c < w.c1 && ok; ++c, ++lc) {
           const int buf = lc & 1;
-          if (!mbar_wait(&acce[buf], ((lc >> 1) & 1) ^ 1, abort_flag)) { ok = false; break; }
+          if (!mbar_wait_warp(&acce[buf], ((lc >> 1) & 1) ^ 1, abort_flag)) { ok = false; break; }
           asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const uint32_t d = tmem + (uint32_t)(buf * ACC_COLS);
           const int kb0 = c * CHB, kb1 = min(kb0 + CHB, g.nk);
           for (int kb = kb0; kb < kb1; ++kb, ++it) {
             const int st = it % ST;
-            if (!mbar_wait(&full[st], (it / ST) & 1, abort_flag)) { ok = false; break; }
+            if (!mbar_wait_warp(&full[st], (it / ST) & 1, abort_flag)) { ok = false; break; }
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             const uint64_t a = sdesc(smem + st * STB), b = sdesc(smem + st * STB + TILE_A);
 #pragma unroll
@@ -360,7 +360,8 @@ __global__ void __launch_bounds__(P_THREADS, 1) k_gemm_f16x3(const __grid_consta
             scol[i * 32 + lane] = sb;
           }
         mild = __all_sync(0xffffffffu, mild);
-        if (!mbar_wait_sleep(&accf[buf], (lc >> 1) & 1, abort_flag)) { ok = false; break; }
+        __syncwarp();   // the lanes' scales are written: every lane reads all of them
+        if (!__all_sync(0xffffffffu, mbar_wait_sleep(&accf[buf], (lc >> 1) & 1, abort_flag))) { ok = false; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
         for (int i = 0; i < EPI_B; ++i)
