@@ -266,10 +266,10 @@ __global__ void __launch_bounds__(SW_THREADS, 1) k_sandwich_tc(const SwArgs a) {
       int k = 0, it = 0;
       bool ok = true;
       while (ok && kp.next(a)) {
-        if (k > 0 && !mbar_wait(d1_empty, (k - 1) & 1, abort_flag)) break;
+        if (k > 0 && !mbar_wait_warp(d1_empty, (k - 1) & 1, abort_flag)) break;
         for (int c = kp.c0(); c < kp.c1(); ++c, ++it) {
           const int st = it % KB_STAGES;
-          if (!mbar_wait(&kb_full[st], (it / KB_STAGES) & 1, abort_flag) || !mbar_wait(ka_full, it & 1, abort_flag)) {
+          if (!mbar_wait_warp(&kb_full[st], (it / KB_STAGES) & 1, abort_flag) || !mbar_wait_warp(ka_full, it & 1, abort_flag)) {
             ok = false;
             break;
           }
@@ -312,17 +312,17 @@ __global__ void __launch_bounds__(SW_THREADS, 1) k_sandwich_tc(const SwArgs a) {
       const int nkk2 = a.k2p / 8;
       const uint32_t ah = tmem + TM_BA + w * 2 * KPAD, al = ah + KPAD;
       const uint32_t d = tmem + TM_D2 + w * TM_D2_STRIDE;
-      bool ok = mbar_wait(ar_full, 0, abort_flag);
+      bool ok = mbar_wait_warp(ar_full, 0, abort_flag);
       PairIter bp;
       bp.start(s_poff);
       int b = 0;
       while (ok && bp.next(a)) {
-        if (b > 0 && !mbar_wait(d2_empty, (b - 1) & 1, abort_flag)) break;
+        if (b > 0 && !mbar_wait_warp(d2_empty, (b - 1) & 1, abort_flag)) break;
         bool first = true;
         for (int q = 0; q < P; ++q) {
           const int qi = P * b + q;   // q blocks run through the two slots in this order
           if ((qi & 1) != w) continue;
-          if (!mbar_wait(&ba_full[w], (qi >> 1) & 1, abort_flag)) {
+          if (!mbar_wait_warp(&ba_full[w], (qi >> 1) & 1, abort_flag)) {
             ok = false;
             break;
           }
