@@ -338,12 +338,10 @@ __global__ void __launch_bounds__(P_THREADS, 1) k_gemm_tf32x3_t(const __grid_con
         // while the previous one is still landing. The slot wait comes first: once the MMAs
         // of k-block it - 2 are done, the fill of it - T_STAGES has landed (those MMAs
         // consumed it), so full[st] is in the phase of k-block it and the parity is exact.
-        if (PAIR ? !mbar_wait(&aempty[as], ((it / NSLOT) & 1) ^ 1, abort_flag)
-                 : !mbar_wait(&empty[st], ((it / T_STAGES) & 1) ^ 1, abort_flag)) {
-          ok = false;
-          break;
-        }
-        if (!mbar_wait(&full[st], (it / T_STAGES) & 1, abort_flag)) { ok = false; break; }
+        const bool ready = (PAIR ? mbar_wait(&aempty[as], ((it / NSLOT) & 1) ^ 1, abort_flag)
+                                 : mbar_wait(&empty[st], ((it / T_STAGES) & 1) ^ 1, abort_flag)) &&
+                           mbar_wait(&full[st], (it / T_STAGES) & 1, abort_flag);
+        if (!__all_sync(0xffffffffu, ready)) { ok = false; break; }   // the stores below are the whole warp's
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint4* row = (const uint4*)(A_f(st) + r * 128);
         float hi[32], lo[32];
@@ -379,7 +377,7 @@ __global__ void __launch_bounds__(P_THREADS, 1) k_gemm_tf32x3_t(const __grid_con
       kslice(tile, kb0, nk);
       for (int kb = 0; kb < nk; ++kb, ++it) {
         const int st = it % T_STAGES;
-        if (!mbar_wait(&full[st], (it / T_STAGES) & 1, abort_flag)) { ok = false; break; }
+        if (!mbar_wait_warp(&full[st], (it / T_STAGES) & 1, abort_flag)) { ok = false; break; }
         uint4* bh = (uint4*)B_hi(st);
         uint4* blo = (uint4*)B_lo(st);
 #pragma unroll 3
@@ -414,7 +412,7 @@ __global__ void __launch_bounds__(P_THREADS, 1) k_gemm_tf32x3_t(const __grid_con
       const int64_t mo = mrow ? (m / g.om.mdiv) * g.om.c0 + (m % g.om.mdiv) * g.om.c1 : 0;
       for (int ch = 0; ch < nch; ++ch, ++lc) {
         const int buf = lc % g.nbuf;
-        if (!mbar_wait(&accf[buf], (lc / g.nbuf) & 1, abort_flag)) { ok = false; break; }
+        if (!mbar_wait_warp(&accf[buf], (lc / g.nbuf) & 1, abort_flag)) { ok = false; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll 1
         for (int cb = 0; cb < BNT; cb += 32) {
