@@ -12,7 +12,7 @@
 //      own scale, so graded matrices lose nothing (a mixed-precision Jacobi preconditioner; Gao,
 //      Ma and Shao 2022).
 //   2. V = V0 (3/2 - V0^T V0 / 2) in FP64, one Newton-Schulz step: orthonormal to FP64 rounding;
-//      M <- M V.
+//      M <- M V, M at unit scale from here on (a power of two, put back on the singular values).
 //   3. G = M^T M gives every remaining angle at once: S_pq = t(G_pp, G_qq, G_pq), the Jacobi
 //      tangents as a skew matrix, and M, V <- M, V exp(S) by matrix products (the first-order
 //      correction of Ogita and Aishima 2020, with the exponential to fourth order so that V stays
@@ -278,10 +278,11 @@ struct SvdState {
   unsigned sweep_rot[2], sweep_big[2];
 };
 
-// the power of two that brings the largest element to [1, 2)
+// the power of two that brings the largest element to [1, 2) (near the ends of FP64: as close as a power
+// of two gets)
 __device__ __forceinline__ double unit_scale(unsigned long long maxbits) {
   const int e = (int)(maxbits >> 52);
-  return maxbits == 0 || e == 0 || e == 0x7FF ? 1.0 : __longlong_as_double((long long)max(2046 - e, 1) << 52);
+  return maxbits == 0 || e == 0x7FF ? 1.0 : __longlong_as_double((long long)max(2046 - e, 1) << 52);
 }
 
 __global__ void k_svd_max(const double* M, int64_t n, SvdState* st) {
@@ -568,10 +569,15 @@ __global__ void __launch_bounds__(32 * J32_B) k_jacobi32_blk(J32Args g) {
 }
 
 // ---------------------------------------------------------------- FP64 refinement
-// G <- 3/2 - G / 2
-__global__ void k_svd_schulz(double* G, int k) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)k * k; e += (int64_t)gridDim.x * blockDim.x)
+// G <- 3/2 - G / 2, and M to unit scale: the angles' test below and that of k_jacobi_svd_blk take fourth
+// powers of the elements, which leave FP64's range for elements beyond 1e+-77 (every pair then passed
+// for orthogonal). A power of two changes no rounding; k_svd_emit puts it back on the singular values.
+__global__ void k_svd_schulz(double* G, double* M, int k, const SvdState* st) {
+  const double sc = unit_scale(st->maxbits);
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)k * k; e += (int64_t)gridDim.x * blockDim.x) {
     G[e] = (e / k == e % k ? 1.5 : 0.0) - 0.5 * G[e];
+    M[e] *= sc;
+  }
 }
 
 // S from G = M^T M (step `it`): S_pq = tan of the Jacobi angle for p < q, S_qp = -S_pq. Pairs that
@@ -673,12 +679,15 @@ __global__ void __launch_bounds__(256) k_svd_norms(const double* M, int k, doubl
   if (lane == 0) sig[j] = sqrt(s);
 }
 
-// U_j = m_j / sigma_j (0 when sigma_j is negligible), written in descending order of sigma (ties by
-// index): sigma[rank], U[:, rank], order[rank] = original column. One block per column. The ranks are
-// those of the bit patterns, a total order (NaN above infinity), so that order is a permutation whatever
-// the input: its entries index V (gather_cols_f64).
+// Rank of a singular value: by bit pattern, a total order (NaN above infinity), so that the order below is
+// a permutation whatever the input. Its entries index V (gather_cols_f64).
 __device__ __forceinline__ unsigned long long order_key(double s) { return (unsigned long long)__double_as_longlong(fabs(s)); }
-__global__ void __launch_bounds__(128) k_svd_emit(const double* M, const double* sig, int k, double* U, double* sigma, int* order) {
+
+// U_j = m_j / sigma_j (0 when sigma_j is negligible), written in descending order of sigma (ties by
+// index): sigma[rank], U[:, rank], order[rank] = original column. st: M is at unit scale (null: as
+// given). One block per column.
+__global__ void __launch_bounds__(128) k_svd_emit(const double* M, const double* sig, int k, double* U, double* sigma, int* order,
+                                                  const SvdState* st) {
   const int j = blockIdx.x;
   const double sj = sig[j];
   const unsigned long long kj = order_key(sj);
@@ -709,7 +718,7 @@ __global__ void __launch_bounds__(128) k_svd_emit(const double* M, const double*
   for (int i = threadIdx.x; i < k; i += 128) U[(int64_t)rank * k + i] = M[(int64_t)j * k + i] * inv;
   if (threadIdx.x == 0) {
     order[rank] = j;
-    sigma[rank] = sj;
+    sigma[rank] = st ? sj / unit_scale(st->maxbits) : sj;
   }
 }
 
@@ -775,11 +784,13 @@ void svd_jacobi_f64(cudaStream_t s, double* Mat, int k, double* U, double* sigma
   ProfToken pt = prof_begin(PROF_FACTOR, s, 0.0, 16.0 * k * k);
   double* M = Mat;
   double* sig = (double*)((char*)ws_dev + 256);
+  const SvdState* unit = nullptr;
   if (!work || k <= kDirect) {
     sweeps_f64(s, Mat, k, V, nullptr, true, ws_dev);
   } else {
     const int64_t kk = (int64_t)k * k;
     SvdState* st = (SvdState*)work;
+    unit = st;
     // state, lists of rotations (16-byte entries), three matrices, the FP32 copy and norms
     double* T1 = (double*)((char*)work + kStateBytes + list_bytes(k));
     double *T2 = T1 + kk, *T3 = T2 + kk;
@@ -826,7 +837,7 @@ void svd_jacobi_f64(cudaStream_t s, double* Mat, int k, double* U, double* sigma
       gemm_simt<double>(s, k, k, k, 1.0, A, ta ? k : 1, ta ? 1 : k, B, k, 1, beta, C, out_colmajor(k, k, k), skip);
     };
     mul(T1, true, T1, T2, 0.0, nullptr);
-    k_svd_schulz<<<grid_of(kk), 256, 0, s>>>(T2, k);
+    k_svd_schulz<<<grid_of(kk), 256, 0, s>>>(T2, Mat, k, st);
     FP_LAUNCH();
     mul(T1, false, T2, V, 0.0, nullptr);
     mul(Mat, false, V, T3, 0.0, nullptr);
@@ -849,7 +860,7 @@ void svd_jacobi_f64(cudaStream_t s, double* Mat, int k, double* U, double* sigma
   }
   k_svd_norms<<<(k + 7) / 8, 256, 0, s>>>(M, k, sig);
   FP_LAUNCH();
-  k_svd_emit<<<k, 128, 0, s>>>(M, sig, k, U, sigma, order);
+  k_svd_emit<<<k, 128, 0, s>>>(M, sig, k, U, sigma, order, unit);
   FP_LAUNCH();
   prof_end(pt, s);
 }
