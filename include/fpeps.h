@@ -58,8 +58,10 @@ typedef enum {
  * a_hi*b_hi + a_hi*b_lo + a_lo*b_hi with FP32 accumulation, every operand split
  * into two 11-bit halves (3 x 2^-22 relative error per product). Small products
  * split into TF32 halves on chip; large ones into FP16 halves with a power-of-two
- * scale per row and 256 terms, where an element more than 2^18 below the largest
- * of its row and 256 terms keeps 2^-40 of that largest instead. BF16X3 (two
+ * scale per row and 256 terms, where an element more than 2^17 below the largest
+ * of its row and 256 terms keeps 2^-39 of that largest instead. Where such elements
+ * can carry a sum (operands graded against each other along it), a large product is
+ * split on chip too. BF16X3 (two
  * 8-bit halves, 3 x 2^-16) is at most as accurate as that and no faster, so a
  * BF16X3 environment runs the same products. The site sandwich is 3xTF32, and the
  * calibration columns and unbiased products run on the FP32 CUDA cores. */

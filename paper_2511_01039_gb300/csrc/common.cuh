@@ -96,14 +96,41 @@ void gemm_simt(cudaStream_t s, int64_t M, int64_t N, int64_t K, T alpha, const T
 
 // Tensor-core GEMM for K-major A [M][lda] and B [N][ldb] (k contiguous), every operand split
 // into two 11-bit halves: products that amortise it run on FP16 planes made beforehand (gemm_tc.cu),
-// the others split into TF32 on chip (gemm_onchip.cu). scratch: its first int is the
-// error word (set to 1 when a bounded wait timed out).
+// the others, and graded operands, split into TF32 on chip (gemm_onchip.cu).
+//
+// Grading, of a product on planes. Of the 256 terms of a row that share a scale, "tiny" ones are not zero
+// and below 2^-17 of the largest (they lose bits), "large" ones at least 2^-9. Such a segment is deep
+// when more than 24 terms are tiny, uneven when more than 17 are not large, narrow when less than 24 are
+// large (fewer of each in a short segment). The sum of a deep segment that is not narrow, against one
+// that is not uneven, is carried by large terms; of two that are not deep, by terms of 20 bits or more.
+// So a product is graded, and left to the on-chip split, when an operand is deep somewhere and the
+// other uneven somewhere, or a segment is both deep and narrow. N(0,1) data has one tiny term in 60000
+// and one in 200 that is not large; rows times singular values, or blocks times small couplings, against
+// such data are not graded.
+// The words hold the mark of the last product that raised them, so a caller clears them once.
+struct Grading {
+  int deep[2], narrow, uneven[2];   // [2]: of A, of B
+};
+__device__ __forceinline__ bool is_graded(const Grading* g, int mark) {
+  const volatile Grading* v = g;
+  return v->narrow == mark || (v->deep[0] == mark && v->uneven[1] == mark) || (v->deep[1] == mark && v->uneven[0] == mark);
+}
+// The first 256 bytes of the scratch, cleared by the caller when it is new: the error word (set to 1
+// when a bounded wait timed out), then a Grading. mark: not zero, another one for every product.
+constexpr size_t kTcHeader = 256;
 bool gemm_tc_supported(int64_t M, int64_t N, int64_t K, int64_t lda, int64_t ldb);
+// settle: graded operands are recomputed on chip, decided on the device (three launches that return at
+// once where there are none). Without it the caller looks at deep and narrow and calls gemm_tc_settle.
 void gemm_tc(cudaStream_t s, int64_t M, int64_t N, int64_t K, const float* A, int64_t lda, const float* B,
-             int64_t ldb, float* C, OutMap om, void* scratch, size_t scratch_bytes);
+             int64_t ldb, float* C, OutMap om, void* scratch, size_t scratch_bytes, int mark, bool settle = true);
+void gemm_tc_settle(cudaStream_t s, int64_t M, int64_t N, int64_t K, const float* A, int64_t lda, const float* B,
+                    int64_t ldb, float* C, OutMap om, void* scratch, size_t scratch_bytes, int mark);
 size_t gemm_tc_scratch_bytes(int64_t M, int64_t N, int64_t K);
-void gemm_onchip(cudaStream_t s, int64_t M, int64_t N, int64_t K, const float* A, int64_t lda, const float* B, int64_t ldb, float* C, OutMap om, void* scratch, size_t scratch_bytes,
-                 bool hold_loads = false);   // hold_loads: self-test of the bounded waits (no loads issued)
+// hold_loads: self-test of the bounded waits (no loads issued); graded: nothing is done unless these
+// operands are (null: always)
+void gemm_onchip(cudaStream_t s, int64_t M, int64_t N, int64_t K, const float* A, int64_t lda, const float* B,
+                 int64_t ldb, float* C, OutMap om, void* scratch, size_t scratch_bytes, bool hold_loads = false,
+                 const Grading* graded = nullptr, int mark = 0);
 size_t gemm_onchip_scratch_bytes(int64_t M, int64_t N, int64_t K);
 // a split operand: planes [rows][k-blocks of 32 terms][32 hi, 32 lo halves], 2^-e of row r in the
 // chunk c of 256 terms at inv[c * inv_stride + r]

@@ -149,6 +149,7 @@ struct Engine : EngineBase {
   void* scr[2] = {nullptr, nullptr};
   size_t scr_n[2] = {0, 0};
   void* tc_scr = nullptr;
+  int tc_mark = 0;          // number of the last tensor-core product (Grading)
   size_t tc_n = 0;
   bool tc_used = false;
 
@@ -210,11 +211,12 @@ struct Engine : EngineBase {
           check_tc();   // keep a recorded timeout before the error word is replaced
           env->al.put(tc_scr);
         }
-        tc_scr = env->al.get(std::max<size_t>(need, 256));
-        tc_n = std::max<size_t>(need, 256);
-        FP_CUDA(cudaMemsetAsync(tc_scr, 0, sizeof(int), s));
+        tc_scr = env->al.get(std::max(need, kTcHeader));
+        tc_n = std::max(need, kTcHeader);
+        FP_CUDA(cudaMemsetAsync(tc_scr, 0, kTcHeader, s));
       }
-      gemm_tc(s, M, N, K, (const float*)A, lda, (const float*)B, ldb, (float*)C, om, tc_scr, tc_n);
+      tc_mark = tc_mark == INT32_MAX ? 1 : tc_mark + 1;
+      gemm_tc(s, M, N, K, (const float*)A, lda, (const float*)B, ldb, (float*)C, om, tc_scr, tc_n, tc_mark);
       tc_used = true;
       return;
     }
@@ -332,9 +334,9 @@ struct Engine : EngineBase {
   // error word of the tensor-core kernels (first int of tc_scr)
   int* tc_err() {
     if (!tc_scr) {
-      tc_scr = env->al.get(256);
-      tc_n = 256;
-      FP_CUDA(cudaMemsetAsync(tc_scr, 0, sizeof(int), s));
+      tc_scr = env->al.get(kTcHeader);
+      tc_n = kTcHeader;
+      FP_CUDA(cudaMemsetAsync(tc_scr, 0, kTcHeader, s));
     }
     tc_used = true;
     return (int*)tc_scr;

@@ -71,6 +71,8 @@ struct TcArgs {
   int nbuf;     // TMEM chunk accumulators: 2 (alternating) when every tile is one chunk or the
                 // running sum is in shared memory (CTA pairs), else 1 (+ running sum in TMEM)
   int hold;     // self-test of the bounded waits: issue no loads, so every consumer times out
+  const Grading* graded;   // nothing is done unless the operands are graded (null: no such test)
+  int mark;
   float* part;  // nsplit > 1: partial results [nsplit][M][N] row-major
 };
 
@@ -147,6 +149,7 @@ __global__ void __launch_bounds__(P_THREADS, 1) k_gemm_tf32x3_t(const __grid_con
   // second set and B, halved per CTA, is converted by warps 6..7 and 17..18.
   constexpr int NAS = PAIR ? 2 : 1;
   constexpr int NBW = PAIR ? 4 : T_NBCONV;
+  if (g.graded && !is_graded(g.graded, g.mark)) return;   // earlier kernels wrote it: the same for a pair
   const uint32_t rank = PAIR ? cluster_rank() : 0;
   const bool issuer = rank == 0;
   // a CTA pair may not split up on a shared early exit, so only single CTAs return here
@@ -516,7 +519,8 @@ __global__ void __launch_bounds__(P_THREADS, 1) k_gemm_tf32x3_t(const __grid_con
 
 // Sum of the K-slice partials in FP64, written through the output map.
 __global__ void k_splitk_reduce(const float* __restrict__ part, int nsplit, int64_t M, int64_t N, OutMap om,
-                                float* __restrict__ C) {
+                                float* __restrict__ C, const Grading* graded, int mark) {
+  if (graded && !is_graded(graded, mark)) return;
   const int64_t tot = M * N;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < tot; e += (int64_t)gridDim.x * blockDim.x) {
     double acc = 0.0;
@@ -642,7 +646,8 @@ size_t gemm_onchip_scratch_bytes(int64_t M, int64_t N, int64_t K) {
 }
 
 void gemm_onchip(cudaStream_t s, int64_t M, int64_t N, int64_t K, const float* A, int64_t lda, const float* B,
-             int64_t ldb, float* C, OutMap om, void* scratch, size_t scratch_bytes, bool hold_loads) {
+                 int64_t ldb, float* C, OutMap om, void* scratch, size_t scratch_bytes, bool hold_loads,
+                 const Grading* graded, int mark) {
   FP_CHECK(scratch && scratch_bytes >= sizeof(int), FPEPS_ERR_ARG, "tensor-core GEMM: scratch");
   FP_CHECK(((uintptr_t)A % 16) == 0 && ((uintptr_t)B % 16) == 0, FPEPS_ERR_ARG, "tensor-core GEMM: operand alignment");
   static bool attr = false;
@@ -664,6 +669,8 @@ void gemm_onchip(cudaStream_t s, int64_t M, int64_t N, int64_t K, const float* A
   g.kch = g.ks <= 2 * KCH_BLOCKS ? g.ks : KCH_BLOCKS;
   g.nbuf = (p.pair || (g.ks + g.kch - 1) / g.kch == 1) ? 2 : 1;
   g.hold = hold_loads ? 1 : 0;
+  g.graded = graded;
+  g.mark = mark;
   g.part = nullptr;
   if (g.nsplit > 1) {
     FP_CHECK(scratch_bytes >= gemm_onchip_scratch_bytes(M, N, K), FPEPS_ERR_ARG, "tensor-core GEMM: scratch too small");
@@ -693,7 +700,7 @@ void gemm_onchip(cudaStream_t s, int64_t M, int64_t N, int64_t K, const float* A
   if (g.nsplit > 1) {
     const int64_t tot = M * N;
     const int rb = (int)std::min<int64_t>((tot + 255) / 256, 152 * 16);
-    k_splitk_reduce<<<rb, 256, 0, s>>>(g.part, g.nsplit, M, N, om, C);
+    k_splitk_reduce<<<rb, 256, 0, s>>>(g.part, g.nsplit, M, N, om, C, graded, mark);
     FP_LAUNCH();
   }
 }

@@ -10,9 +10,12 @@
 // The split. Every FP32 element is written as x 2^e = hi + lo with hi, lo FP16 (11 significant
 // bits each) and one power of two 2^e per row and segment of 256 terms, chosen so that the
 // segment's largest element lies in [2^14, 2^15). hi + lo then carries 22 bits of every element
-// within 2^-18 of its segment's largest (|x - hi - lo| <= 2^-22 |x|, the same as a split into two
-// TF32 numbers) and 2^-40 of the largest for smaller ones. The product is
+// within 2^-17 of its segment's largest (|x - hi - lo| <= 2^-22 |x|, the same as a split into two
+// TF32 numbers; lo is a multiple of 2^-24, so smaller ones keep 2^-39 of the largest). The product is
 // a_lo b_hi + a_hi b_lo + a_hi b_hi, FP16 x FP16 being exact in the FP32 accumulator.
+// The smaller ones matter where the operands are graded against each other (A falls along k where B
+// rises, or A's large terms meet zeros of B): they carry the sum. Such products are found by the
+// splitting pass (Grading, common.cuh) and computed again with the on-chip split.
 // Why FP16 and not TF32 halves: an FP16 MMA does twice the terms of a TF32 MMA of the same cost,
 // and hi and lo together take the four bytes of the FP32 element, so both operands are split
 // once, in one streaming pass (k_split_planes), and the GEMM moves no more bytes than before.
@@ -75,17 +78,35 @@ struct SplitOp {
   float* inv;       // [nseg][rows]: 2^-e
 };
 
+// Counts of a segment for Grading, by the whole warp: its elements are src[0 .. len), largest top (finite,
+// not zero). large: at least 2^-9 of it, tiny: not zero and below 2^-17.
+struct Terms {
+  int large, tiny;
+};
+__device__ __noinline__ Terms count_terms(const float* src, int len, float top) {
+  const float high = 0x1p-9f * top, low = 0x1p-17f * top;
+  int nl = 0, nt = 0;
+  for (int i = threadIdx.x % 32; i < len; i += 32) {
+    const float x = fabsf(src[i]);
+    nl += x >= high;
+    nt += x != 0.f && x < low;
+  }
+  return Terms{__reduce_add_sync(0xffffffffu, nl), __reduce_add_sync(0xffffffffu, nt)};
+}
+
 // One warp per (row, segment): 8 elements per lane, the segment's largest magnitude by shuffles,
-// one read and one write of four bytes per element (HBM-bound). An infinite or NaN element keeps
-// its value in hi (lo becomes NaN), so non-finite input still gives non-finite output.
-__global__ void __launch_bounds__(256) k_split_planes(SplitOp a, SplitOp b, int64_t K, int64_t nk, int64_t nseg) {
+// one read and one write of four bytes per element (HBM-bound, with two thirds of the issue slots and
+// all warps of an SM in flight: 32 registers at most). An infinite or NaN element keeps its value in hi (lo
+// becomes NaN), so non-finite input still gives non-finite output. The terms of a segment are counted
+// only where one of them is tiny.
+__global__ void __launch_bounds__(256, 8) k_split_planes(SplitOp a, SplitOp b, int64_t K, unsigned nk, unsigned nseg, Grading* gr, int mark) {
   const int lane = threadIdx.x % 32;
-  const int64_t wa = a.rows * nseg, tot = wa + b.rows * nseg;
-  const int64_t nw = (int64_t)gridDim.x * (blockDim.x / 32);
-  for (int64_t w = blockIdx.x * (int64_t)(blockDim.x / 32) + threadIdx.x / 32; w < tot; w += nw) {
+  const unsigned wa = (unsigned)a.rows * nseg, tot = wa + (unsigned)b.rows * nseg;   // a segment takes 1 KB: 32 bits do
+  const unsigned nw = gridDim.x * (blockDim.x / 32);
+  for (unsigned w = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32; w < tot; w += nw) {
     const SplitOp& o = w < wa ? a : b;
-    const int64_t v = w < wa ? w : w - wa, row = v / nseg, seg = v % nseg;
-    const int64_t k = seg * SEG + lane * 8;
+    const unsigned v = w < wa ? w : w - wa, row = v / nseg, seg = v - row * nseg;
+    const int64_t k = (int64_t)seg * SEG + lane * 8;
     const float* src = o.x + row * o.ld + k;
     float f[8];
     if (k + 8 <= K) {   // rows start on 16-byte boundaries and k is a multiple of 8
@@ -97,8 +118,12 @@ __global__ void __launch_bounds__(256) k_split_planes(SplitOp a, SplitOp b, int6
       for (int i = 0; i < 8; ++i) f[i] = k + i < K ? src[i] : 0.f;
     }
     float mx = 0.f;
+    uint32_t mn = ~0u;   // smallest magnitude that is not zero, twice its bits less one
 #pragma unroll
-    for (int i = 0; i < 8; ++i) mx = fmaxf(mx, fabsf(f[i]));
+    for (int i = 0; i < 8; ++i) {
+      mx = fmaxf(mx, fabsf(f[i]));
+      mn = min(mn, 2 * __float_as_uint(f[i]) - 1);
+    }
     const uint32_t mb = __reduce_max_sync(0xffffffffu, __float_as_uint(mx));   // largest magnitude of the segment
     const int ex = (int)(mb >> 23);
     const int e = mb == 0 || ex == 255 ? 0 : min(141 - ex, 126);
@@ -113,13 +138,44 @@ __global__ void __launch_bounds__(256) k_split_planes(SplitOp a, SplitOp b, int6
       h2[i] = *(const uint32_t*)&h;
       l2[i] = *(const uint32_t*)&l;
     }
-    const int64_t kb = k / BK;
+    const unsigned kb = seg * CHB + lane / 4;
     if (kb < nk) {   // the last k-block is padded with zeros
-      __half* dst = o.planes + (row * nk + kb) * (2 * BK) + (lane % 4) * 8;
+      __half* dst = o.planes + ((int64_t)row * nk + kb) * (2 * BK) + (lane % 4) * 8;
       *(uint4*)dst = make_uint4(h2[0], h2[1], h2[2], h2[3]);
       *(uint4*)(dst + BK) = make_uint4(l2[0], l2[1], l2[2], l2[3]);
     }
-    if (lane == 0) o.inv[seg * o.rows + row] = __int_as_float((127 - e) << 23);
+    if (lane == 0) o.inv[(int64_t)seg * o.rows + row] = __int_as_float((127 - e) << 23);
+    const float top = __uint_as_float(mb);
+    if (__any_sync(0xffffffffu, mn < 2 * __float_as_uint(0x1p-17f * top) - 1) && mb != 0 && ex != 255) {
+      const int len = (int)min((int64_t)SEG, K - (int64_t)seg * SEG);
+      const Terms n = count_terms(src - lane * 8, len, top);
+      if (lane == 0 && n.tiny > min(24, 2 + len / 8)) {
+        gr->deep[w < wa ? 0 : 1] = mark;
+        if (n.large < 3 * len / 32) gr->narrow = mark;
+      }
+    }
+  }
+}
+
+// The second half of the test, over the FP32 operands, only when the other operand is deep
+__global__ void __launch_bounds__(256) k_uneven(SplitOp a, SplitOp b, int64_t K, unsigned nseg, Grading* gr, int mark) {
+  const bool need[2] = {*(volatile int*)&gr->deep[1] == mark, *(volatile int*)&gr->deep[0] == mark};
+  if (!need[0] && !need[1]) return;
+  const int lane = threadIdx.x % 32;
+  const int64_t wa = a.rows * (int64_t)nseg, tot = wa + b.rows * (int64_t)nseg;
+  for (int64_t w = blockIdx.x * (int64_t)(blockDim.x / 32) + threadIdx.x / 32; w < tot; w += (int64_t)gridDim.x * (blockDim.x / 32)) {
+    const int which = w < wa ? 0 : 1;
+    if (!need[which] || *(volatile int*)&gr->uneven[which] == mark) continue;
+    const SplitOp& o = which ? b : a;
+    const int64_t v = which ? w - wa : w, row = v / nseg, seg = v % nseg;
+    const int len = (int)min((int64_t)SEG, K - seg * SEG);
+    const float* src = o.x + row * o.ld + seg * SEG;
+    float mx = 0.f;
+    for (int i = lane; i < len; i += 32) mx = fmaxf(mx, fabsf(src[i]));
+    const uint32_t mb = __reduce_max_sync(0xffffffffu, __float_as_uint(mx));
+    if (mb == 0 || (mb >> 23) == 255) continue;   // zeros: exact; not finite: so is the result
+    const Terms n = count_terms(src, len, __uint_as_float(mb));
+    if (lane == 0 && n.large < len - 1 - len / 16) gr->uneven[which] = mark;
   }
 }
 
@@ -699,7 +755,8 @@ int64_t panel_of(int64_t M, int64_t N, int64_t K) {
   return ((K + np - 1) / np + SEG - 1) / SEG * SEG;   // whole scale segments
 }
 
-// scratch: error word, pieces of cut tiles, then the split operands and their scales
+// scratch: header, pieces of cut tiles, then the split operands and their scales; the on-chip split of
+// graded operands uses the same bytes after them
 size_t part_bytes(const Plan& p) {
   return p.full < p.mt * p.nt ? up256((size_t)2 * p.slots * p.bn * BM * (p.pair ? 2 : 1) * 4) : 0;
 }
@@ -707,6 +764,8 @@ size_t split_bytes(int64_t rows, int64_t K) {
   const int64_t nk = (K + BK - 1) / BK, nch = (nk + CHB - 1) / CHB;
   return up256((size_t)rows * nk * ROWB) + up256((size_t)rows * nch * 4);
 }
+
+Grading* grading_of(void* scratch) { return (Grading*)((int*)scratch + 4); }
 
 void run_planes(cudaStream_t s, int64_t M, int64_t N, int64_t K, const SplitMat& A, const SplitMat& B, float* C, OutMap om,
                 void* scratch, bool accumulate, bool hold) {
@@ -726,7 +785,7 @@ void run_planes(cudaStream_t s, int64_t M, int64_t N, int64_t K, const SplitMat&
   const int out = om.c3 != 1 ? LANES : granules ? ROWS_BULK : ROWS;
   g.inva = A.inv; g.invb = B.inv;
   g.sca = A.inv_stride; g.scb = B.inv_stride;
-  g.part = (float*)((char*)scratch + 256);
+  g.part = (float*)((char*)scratch + kTcHeader);
   g.bn = p.bn;
   g.mt = (int)p.mt; g.nt = (int)p.nt;
   g.m_fast = g.mt <= g.nt ? 1 : 0;
@@ -755,12 +814,13 @@ bool gemm_tc_supported(int64_t M, int64_t N, int64_t K, int64_t lda, int64_t ldb
 size_t gemm_tc_scratch_bytes(int64_t M, int64_t N, int64_t K) {
   if (!on_planes(M, N, K)) return gemm_onchip_scratch_bytes(M, N, K);
   const int64_t kp = panel_of(M, N, K), last = K - (K - 1) / kp * kp;
-  return 256 + std::max(part_bytes(plan_of(M, N, std::min(kp, K))), part_bytes(plan_of(M, N, last))) +
-         split_bytes(M, std::min(kp, K)) + split_bytes(N, std::min(kp, K));
+  return std::max(gemm_onchip_scratch_bytes(M, N, K),
+                  kTcHeader + std::max(part_bytes(plan_of(M, N, std::min(kp, K))), part_bytes(plan_of(M, N, last))) +
+                      split_bytes(M, std::min(kp, K)) + split_bytes(N, std::min(kp, K)));
 }
 
 void gemm_tc(cudaStream_t s, int64_t M, int64_t N, int64_t K, const float* A, int64_t lda, const float* B,
-             int64_t ldb, float* C, OutMap om, void* scratch, size_t scratch_bytes) {
+             int64_t ldb, float* C, OutMap om, void* scratch, size_t scratch_bytes, int mark, bool settle) {
   FP_CHECK(((uintptr_t)A % 16) == 0 && ((uintptr_t)B % 16) == 0, FPEPS_ERR_ARG, "tensor-core GEMM: operand alignment");
   FP_CHECK(scratch && scratch_bytes >= gemm_tc_scratch_bytes(M, N, K), FPEPS_ERR_ARG, "tensor-core GEMM: scratch too small");
   ProfToken pt = prof_begin(PROF_GEMM_TC, s, 2.0 * M * N * K, 4.0 * ((double)M * K + (double)N * K + (double)M * N));
@@ -772,15 +832,26 @@ void gemm_tc(cudaStream_t s, int64_t M, int64_t N, int64_t K, const float* A, in
   const int64_t kp = panel_of(M, N, K);
   for (int64_t k0 = 0; k0 < K; k0 += kp) {
     const int64_t k = std::min(kp, K - k0), nk = (k + BK - 1) / BK, nch = (nk + CHB - 1) / CHB;
-    char* base = (char*)scratch + 256 + part_bytes(plan_of(M, N, k));
+    char* base = (char*)scratch + kTcHeader + part_bytes(plan_of(M, N, k));
     SplitOp oa{A + k0, M, lda, (__half*)base, (float*)(base + up256((size_t)M * nk * ROWB))};
     base += split_bytes(M, k);
     SplitOp ob{B + k0, N, ldb, (__half*)base, (float*)(base + up256((size_t)N * nk * ROWB))};
-    k_split_planes<<<(unsigned)std::min<int64_t>(((M + N) * nch + 7) / 8, 152 * 32), 256, 0, s>>>(oa, ob, k, nk, nch);
+    k_split_planes<<<(unsigned)std::min<int64_t>(((M + N) * nch + 7) / 8, 152 * 32), 256, 0, s>>>(oa, ob, k, (unsigned)nk, (unsigned)nch,
+                                                                                                         grading_of(scratch), mark);
     FP_LAUNCH();
     run_planes(s, M, N, k, SplitMat{oa.planes, oa.inv, M}, SplitMat{ob.planes, ob.inv, N}, C, om, scratch, k0 > 0, false);
   }
+  if (settle) gemm_tc_settle(s, M, N, K, A, lda, B, ldb, C, om, scratch, scratch_bytes, mark);
   prof_end(pt, s);
+}
+
+void gemm_tc_settle(cudaStream_t s, int64_t M, int64_t N, int64_t K, const float* A, int64_t lda, const float* B,
+                    int64_t ldb, float* C, OutMap om, void* scratch, size_t scratch_bytes, int mark) {
+  if (!on_planes(M, N, K)) return;
+  const SplitOp oa{A, M, lda, nullptr, nullptr}, ob{B, N, ldb, nullptr, nullptr};
+  k_uneven<<<152, 256, 0, s>>>(oa, ob, K, (unsigned)((K + SEG - 1) / SEG), grading_of(scratch), mark);
+  FP_LAUNCH();
+  gemm_onchip(s, M, N, K, A, lda, B, ldb, C, om, scratch, scratch_bytes, false, grading_of(scratch), mark);
 }
 
 void gemm_tc_hold(cudaStream_t s, int64_t M, int64_t N, int64_t K, void* planes, float* C, void* scratch) {
