@@ -72,6 +72,7 @@ void* Allocator::get(size_t bytes) {
     p = a.alloc(a.ctx, bytes, (void*)stream);
     if (!p) {
       trim_pools();
+      if (reclaim) reclaim();
       p = a.alloc(a.ctx, bytes, (void*)stream);
     }
     if (!p) throw Error{FPEPS_ERR_OOM, "allocator returned NULL for " + std::to_string(bytes) + " bytes"};
@@ -81,6 +82,7 @@ void* Allocator::get(size_t bytes) {
   if (e == cudaErrorMemoryAllocation) {
     cudaGetLastError();
     trim_pools();
+    if (reclaim) reclaim();
     e = cudaMallocAsync(&p, bytes, stream);
   }
   if (e == cudaErrorMemoryAllocation) {
@@ -748,9 +750,15 @@ fpeps_status fpeps_gemm_f32(int32_t mode, int64_t M, int64_t N, int64_t K, const
     if (mode != FPEPS_TF32X3 && mode != FPEPS_BF16X3) throw Error{FPEPS_ERR_UNSUPPORTED, "mode"};
     if (!fpeps::gemm_tc_supported(M, N, K, lda, ldb) || ((uintptr_t)A % 16) || ((uintptr_t)B % 16))
       throw Error{FPEPS_ERR_UNSUPPORTED, "shape not supported by the tensor-core kernel"};
-    const size_t sb = fpeps::gemm_tc_scratch_bytes(M, N, K);
+    size_t sb = fpeps::gemm_tc_scratch_bytes(M, N, K);
     int* err = nullptr;
-    FP_CUDA(cudaMallocFromPoolAsync((void**)&err, sb, fpeps::scratch_pool(), s));
+    cudaError_t e = cudaMallocFromPoolAsync((void**)&err, sb, fpeps::scratch_pool(), s);
+    if (e == cudaErrorMemoryAllocation) {   // no room for planes: the on-chip split needs little
+      cudaGetLastError();
+      sb = fpeps::gemm_onchip_scratch_bytes(M, N, K);
+      e = cudaMallocFromPoolAsync((void**)&err, sb, fpeps::scratch_pool(), s);
+    }
+    FP_CUDA(e);
     FP_CUDA(cudaMemsetAsync(err, 0, fpeps::kTcHeader, s));
     fpeps::gemm_tc(s, M, N, K, A, lda, B, ldb, C, om, err, sb, 1, false);
     static thread_local fpeps::StatusWords words;

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <functional>
 #include <string>
 #include <vector>
 
@@ -58,6 +59,7 @@ struct Allocator {
   fpeps_allocator a{};
   bool has = false;
   cudaStream_t stream = nullptr;
+  std::function<void()> reclaim;   // gives back what its owner can do without, before an allocation fails
   void* get(size_t bytes);
   void put(void* p);
 };
@@ -119,7 +121,8 @@ __device__ __forceinline__ bool is_graded(const Grading* g, int mark) {
 // when a bounded wait timed out), then a Grading. mark: not zero, another one for every product.
 constexpr size_t kTcHeader = 256;
 bool gemm_tc_supported(int64_t M, int64_t N, int64_t K, int64_t lda, int64_t ldb);
-// settle: graded operands are recomputed on chip, decided on the device (three launches that return at
+// Scratch of fewer bytes than gemm_tc_scratch_bytes, but at least gemm_onchip_scratch_bytes, sends the
+// product to the on-chip split. settle: graded operands are recomputed on chip, decided on the device (three launches that return at
 // once where there are none). Without it the caller looks at deep and narrow and calls gemm_tc_settle.
 void gemm_tc(cudaStream_t s, int64_t M, int64_t N, int64_t K, const float* A, int64_t lda, const float* B,
              int64_t ldb, float* C, OutMap om, void* scratch, size_t scratch_bytes, int mark, bool settle = true);

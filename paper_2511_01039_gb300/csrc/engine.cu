@@ -151,6 +151,7 @@ struct Engine : EngineBase {
   void* tc_scr = nullptr;
   int tc_mark = 0;          // number of the last tensor-core product (Grading)
   size_t tc_n = 0;
+  size_t tc_refused = SIZE_MAX;   // smallest tensor-core scratch that the allocator refused
   bool tc_used = false;
 
   // optional per-phase wall times (FPEPS_TRACE=1): synchronises around each phase
@@ -177,8 +178,10 @@ struct Engine : EngineBase {
   explicit Engine(fpeps_env* e) : env(e), s(e->stream), mode(e->cfg.prec) {
     if (const char* b = getenv("FPEPS_CHUNK_ELEMS")) budget_elems = (size_t)atoll(b);
     if (const char* t = getenv("FPEPS_TRACE")) trace = atoi(t) != 0;
+    env->al.reclaim = [this] { reclaim_tc_scratch(); };
   }
   ~Engine() override {
+    env->al.reclaim = nullptr;
     for (int i = 0; i < 2; ++i)
       if (scr[i]) env->al.put(scr[i]);
     if (tc_scr) env->al.put(tc_scr);
@@ -205,16 +208,7 @@ struct Engine : EngineBase {
     if (sizeof(T) == 4 && (mode == FPEPS_TF32X3 || mode == FPEPS_BF16X3) && !simt_only &&
         gemm_tc_supported(M, N, K, lda, ldb) &&
         ((uintptr_t)A % 16) == 0 && ((uintptr_t)B % 16) == 0) {
-      size_t need = gemm_tc_scratch_bytes(M, N, K);
-      if (!tc_scr || tc_n < need) {
-        if (tc_scr) {
-          check_tc();   // keep a recorded timeout before the error word is replaced
-          env->al.put(tc_scr);
-        }
-        tc_scr = env->al.get(std::max(need, kTcHeader));
-        tc_n = std::max(need, kTcHeader);
-        FP_CUDA(cudaMemsetAsync(tc_scr, 0, kTcHeader, s));
-      }
+      tc_scratch(gemm_tc_scratch_bytes(M, N, K), gemm_onchip_scratch_bytes(M, N, K));
       tc_mark = tc_mark == INT32_MAX ? 1 : tc_mark + 1;
       gemm_tc(s, M, N, K, (const float*)A, lda, (const float*)B, ldb, (float*)C, om, tc_scr, tc_n, tc_mark);
       tc_used = true;
@@ -331,6 +325,37 @@ struct Engine : EngineBase {
     const T* Et = nullptr;
   };
 
+  // Scratch of the tensor-core products: `want` bytes, or `least` (the on-chip split's) where the
+  // allocator refuses them. A refused size is not asked for again before the next row.
+  void tc_scratch(size_t want, size_t least) {
+    if (want >= tc_refused) want = least;
+    if (tc_scr && tc_n >= want) return;
+    drop_tc_scratch();
+    try {
+      tc_scr = env->al.get(want);
+    } catch (const Error& e) {
+      if (e.st != FPEPS_ERR_OOM || want == least) throw;
+      tc_refused = want;
+      want = least;
+      tc_scr = env->al.get(want);
+    }
+    tc_n = want;
+    FP_CUDA(cudaMemsetAsync(tc_scr, 0, kTcHeader, s));
+  }
+  // what an allocation that fails elsewhere can have: the planes
+  void reclaim_tc_scratch() {
+    if (!tc_scr || tc_n == kTcHeader) return;
+    tc_refused = std::min(tc_refused, tc_n);
+    drop_tc_scratch();
+  }
+  void drop_tc_scratch() {
+    if (!tc_scr) return;
+    check_tc();   // a recorded timeout is reported before the error word goes
+    tc_used = false;
+    env->al.put(tc_scr);
+    tc_scr = nullptr;
+    tc_n = 0;
+  }
   // error word of the tensor-core kernels (first int of tc_scr)
   int* tc_err() {
     if (!tc_scr) {
@@ -819,6 +844,7 @@ struct Engine : EngineBase {
     const int chi = e->cfg.chi;
     ensure_sandwich(e, e->layer, row);
     flops = 0.0;
+    tc_refused = SIZE_MAX;
     trunc_num = trunc_den = 0.0;
     for (double& v : ph) v = 0.0;
     const auto t_start = std::chrono::steady_clock::now();
@@ -1741,6 +1767,7 @@ struct Engine : EngineBase {
     const int row = e->staged_row;
     FP_CHECK(row > 0, FPEPS_ERR_STATE, "no staged row");
     ensure_sandwich(e, e->layer, row);
+    tc_refused = SIZE_MAX;
     Arena ar = arena();
     const bool right = op >= 2;
     Site st = make_site(ar, row, c, !right, right);
