@@ -190,6 +190,8 @@ struct Engine : EngineBase {
   T* scratch(int i, size_t n) {
     if (scr_n[i] < n) {
       if (scr[i]) env->al.put(scr[i]);
+      scr[i] = nullptr;   // stays so if the larger block is refused
+      scr_n[i] = 0;
       scr[i] = env->al.get(n * sizeof(T));
       scr_n[i] = n;
     }

@@ -15,7 +15,7 @@ class _Bounded:
     def __init__(self, fp, limit=None):
         import torch
         self.inner = fp.TorchAllocator(torch.device("cuda", torch.cuda.current_device()))
-        self.limit, self.live, self.held, self.peak, self.refused = limit, {}, 0, 0, 0
+        self.limit, self.live, self.held, self.peak, self.refused, self.stray = limit, {}, 0, 0, 0, 0
         self._a, self._f = fp.ALLOC_FN(self._alloc), fp.FREE_FN(self._free)
         self.struct = fp.fpeps_allocator(None, self._a, self._f)
 
@@ -30,6 +30,9 @@ class _Bounded:
         return p
 
     def _free(self, ctx, ptr, stream):
+        if ptr not in self.live:
+            self.stray += 1   # not a block of ours, or given back twice
+            return
         self.held -= self.live.pop(ptr)
         self.inner._free(ctx, ptr, stream)
 
@@ -104,3 +107,34 @@ def test_row_without_room_for_the_planes():
     tight = _Bounded(fp, peak - (16 << 20))   # the copies of this size take some 50 MB
     got, _ = row(tight)
     assert tight.refused and abs(got - want) < 1e-4
+
+
+def test_refused_growth_leaves_the_handle_usable():
+    """A call that runs out of memory while an intermediate grows gives every block back once, and the
+    handle computes the smaller call as before."""
+    from paper_2511_01039_gb300 import fpeps as fp
+    from paper_2511_01039_gb300 import workloads as WL
+    chi = 60
+    al = _Bounded(fp)
+    h = _handle(fp, al, 3, 3, chi)
+    g = np.random.default_rng(3)
+    bnd = [g.standard_normal(s, dtype=np.float32) for s in ((1, B, chi), (chi, B, chi), (chi, B, 1))]
+    fp.fpeps_import_boundary(h, WL.boundary_blob(bnd, 1, 1, 4), 1, 1)
+    fp.fpeps_absorb_row(h, 1, 1)
+    e = g.standard_normal((chi, chi, B), dtype=np.float32)
+    x = g.standard_normal((80, chi, B), dtype=np.float32)
+    call = lambda k: fp.fpeps_apply_theta_op(h, 0, 1, e, x[:k], (chi, B), 4)
+    want = call(2)
+    big = []
+    for room in range(8, 200, 8):   # MB beyond what is held: the refusal falls on one block after the other
+        al.limit = al.held + (room << 20)
+        try:
+            big.append(call(80))
+            break
+        except fp.FpepsError as err:
+            assert err.status == 3
+        al.limit = None
+        assert np.array_equal(call(2), want)
+    assert al.refused and al.stray == 0
+    fp.fpeps_env_destroy(h)
+    assert al.stray == 0 and not al.live
