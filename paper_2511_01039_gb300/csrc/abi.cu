@@ -1,5 +1,7 @@
 // C ABI of libfpeps: environment lifecycle, the row state machine and
 // checkpoints. Every entry point converts internal errors to fpeps_status.
+#include <cuda.h>
+
 #include <algorithm>
 #include <atomic>
 #include <cmath>
@@ -15,55 +17,87 @@ using fpeps::Error;
 
 namespace fpeps {
 
-// Scratch of the calls without a handle (fpeps_gemm_f32): a pool of the library's own per device,
+uint64_t context_id() {
+  using GetCurrent = CUresult (*)(CUcontext*);
+  using GetId = CUresult (*)(CUcontext, unsigned long long*);
+  static GetCurrent current = nullptr;
+  static GetId id_of = nullptr;
+  static std::once_flag once;
+  std::call_once(once, [] {
+    cudaDriverEntryPointQueryResult q;
+    void* p = nullptr;
+    if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &p, 12000, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess)
+      current = (GetCurrent)p;
+    if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &p, 12000, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess)
+      id_of = (GetId)p;
+  });
+  FP_CHECK(current && id_of, FPEPS_ERR_CUDA, "cuCtxGetId unavailable");
+  for (int t = 0;; ++t) {
+    CUcontext ctx = nullptr;
+    unsigned long long id = 0;
+    if (current(&ctx) == CUDA_SUCCESS && ctx && id_of(ctx, &id) == CUDA_SUCCESS) return id;
+    FP_CHECK(t == 0, FPEPS_ERR_CUDA, "no current CUDA context");
+    FP_CUDA(cudaFree(nullptr));
+  }
+}
+
+// Scratch of the calls without a handle (fpeps_gemm_f32): a pool of the library's own per context,
 // shared by all threads and streams (stream-ordered). The default pool hands its memory back at
 // every synchronisation, and mapping half a gigabyte again costs the next call a millisecond; this
-// one keeps up to kKeep bytes, which trim_pools() gives back (when an environment is destroyed or an
+// one keeps up to kKeep bytes, which trim_pool() gives back (when an environment is destroyed or an
 // allocation fails).
 namespace {
 constexpr uint64_t kKeep = 640ull << 20;
-std::mutex g_pool_mu;
-std::map<int, cudaMemPool_t> g_pools;
+PerContext<cudaMemPool_t> g_pools;
 }  // namespace
 
 static cudaMemPool_t scratch_pool() {
-  int dev = 0;
-  FP_CUDA(cudaGetDevice(&dev));
-  std::lock_guard<std::mutex> lk(g_pool_mu);
-  auto it = g_pools.find(dev);
-  if (it != g_pools.end()) return it->second;
-  cudaMemPoolProps pr = {};
-  pr.allocType = cudaMemAllocationTypePinned;
-  pr.location.type = cudaMemLocationTypeDevice;
-  pr.location.id = dev;
-  cudaMemPool_t pool;
-  FP_CUDA(cudaMemPoolCreate(&pool, &pr));
-  uint64_t keep = kKeep;
-  FP_CUDA(cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep));
-  g_pools[dev] = pool;
-  return pool;
+  return g_pools.get([] {
+    int dev = 0;
+    FP_CUDA(cudaGetDevice(&dev));
+    cudaMemPoolProps pr = {};
+    pr.allocType = cudaMemAllocationTypePinned;
+    pr.location.type = cudaMemLocationTypeDevice;
+    pr.location.id = dev;
+    cudaMemPool_t pool;
+    FP_CUDA(cudaMemPoolCreate(&pool, &pr));
+    uint64_t keep = kKeep;
+    FP_CUDA(cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep));
+    return pool;
+  });
 }
 
-// Pinned words for the status that a call without a handle reads back, one set per thread: into pageable
-// memory the copy goes through the driver's staging (1000 x 2000 x 500: 46.0 -> 43.5 us a call). Null if
-// they can't be had: words on the stack serve then.
+// Pinned words for the status that a call without a handle reads back, one set per thread and context:
+// into pageable memory the copy goes through the driver's staging (1000 x 2000 x 500: 46.0 -> 43.5 us a
+// call). Null if they can't be had: words on the stack serve then.
 struct StatusWords {
   static constexpr int N = 8;   // error word, grading (kTcHeader's first words)
-  int* p = nullptr;
-  StatusWords() {
-    if (cudaHostAlloc((void**)&p, N * sizeof(int), cudaHostAllocPortable) != cudaSuccess) {
+  std::map<uint64_t, int*> words;
+  int* get() {
+    auto it = words.find(context_id());
+    if (it != words.end()) return it->second;
+    int* p = nullptr;
+    if (cudaHostAlloc((void**)&p, N * sizeof(int), cudaHostAllocDefault) != cudaSuccess) {
       cudaGetLastError();
-      p = nullptr;
+      return nullptr;
     }
+    return words[context_id()] = p;
   }
-  ~StatusWords() {
-    if (p) cudaFreeHost(p);
+  ~StatusWords() {   // the current context's; another one's may be gone, with its words
+    try {
+      if (!words.empty()) {
+        auto it = words.find(context_id());
+        if (it != words.end()) cudaFreeHost(it->second);
+      }
+    } catch (const Error&) {
+    }
   }
 };
 
-static void trim_pools() {
-  std::lock_guard<std::mutex> lk(g_pool_mu);
-  for (auto& p : g_pools) cudaMemPoolTrimTo(p.second, 0);
+// the scratch pool of the current context
+static void trim_pool() {
+  cudaMemPool_t pool;
+  if (g_pools.peek(pool)) cudaMemPoolTrimTo(pool, 0);
 }
 
 void* Allocator::get(size_t bytes) {
@@ -71,7 +105,7 @@ void* Allocator::get(size_t bytes) {
   if (has) {
     p = a.alloc(a.ctx, bytes, (void*)stream);
     if (!p) {
-      trim_pools();
+      trim_pool();
       if (reclaim) reclaim();
       p = a.alloc(a.ctx, bytes, (void*)stream);
     }
@@ -81,7 +115,7 @@ void* Allocator::get(size_t bytes) {
   cudaError_t e = cudaMallocAsync(&p, bytes, stream);
   if (e == cudaErrorMemoryAllocation) {
     cudaGetLastError();
-    trim_pools();
+    trim_pool();
     if (reclaim) reclaim();
     e = cudaMallocAsync(&p, bytes, stream);
   }
@@ -653,7 +687,7 @@ void fpeps_env_destroy(fpeps_env* env) {
     if (env->stream || !env->al.has) cudaStreamSynchronize(env->stream);
     if (env->h_info) cudaFreeHost(env->h_info);
     if (env->h_scal) cudaFreeHost(env->h_scal);
-    fpeps::trim_pools();
+    fpeps::trim_pool();
   } catch (...) {
   }
   delete env;
@@ -763,7 +797,8 @@ fpeps_status fpeps_gemm_f32(int32_t mode, int64_t M, int64_t N, int64_t K, const
     fpeps::gemm_tc(s, M, N, K, A, lda, B, ldb, C, om, err, sb, 1, false);
     static thread_local fpeps::StatusWords words;
     int on_stack[fpeps::StatusWords::N] = {};
-    int* const h = words.p ? words.p : on_stack;
+    int* const pinned = words.get();
+    int* const h = pinned ? pinned : on_stack;
     FP_CUDA(cudaMemcpyAsync(h, err, sizeof(on_stack), cudaMemcpyDeviceToHost, s));
     FP_CUDA(cudaStreamSynchronize(s));
     if (!*h && (h[4] || h[5] || h[6])) {   // deep or narrow segments: the rest of the test, and the on-chip split if graded

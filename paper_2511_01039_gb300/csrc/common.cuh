@@ -8,6 +8,7 @@
 #include <string>
 #include <vector>
 
+#include "context.cuh"
 #include "fpeps.h"
 
 namespace fpeps {

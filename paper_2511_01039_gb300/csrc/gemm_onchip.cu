@@ -581,25 +581,25 @@ static int nsplit_of(int64_t tiles, int64_t K, int sms) {
   return best;
 }
 
-static int sm_count() {
-  static int sms = 0;
-  if (!sms) {
-    int dev = 0;
-    FP_CUDA(cudaGetDevice(&dev));
-    FP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  }
-  return sms;
-}
-
-// CTA pairs the GPU holds at once (clusters of two CTAs, one CTA per SM); 0 if
-// the pair kernel cannot be launched
-static int pair_slots() {
-  static int n = -1;
-  if (n < 0) {
+// SMs, and CTA pairs the GPU holds at once (clusters of two CTAs, one CTA per SM; 0 if
+// the pair kernel cannot be launched). Asking for them also prepares the kernels for
+// launches in this context.
+struct Limits {
+  int sms, pairs;
+};
+static Limits limits() {
+  static PerContext<Limits> per;
+  return per.get([] {
+    FP_CUDA(cudaFuncSetAttribute(k_gemm_tf32x3_t<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 t_smem_bytes<false>()));
     FP_CUDA(cudaFuncSetAttribute(k_gemm_tf32x3_t<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  t_smem_bytes<true>()));
+    int dev = 0;
+    Limits l{0, 0};
+    FP_CUDA(cudaGetDevice(&dev));
+    FP_CUDA(cudaDeviceGetAttribute(&l.sms, cudaDevAttrMultiProcessorCount, dev));
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(sm_count() & ~1));
+    cfg.gridDim = dim3((unsigned)(l.sms & ~1));
     cfg.blockDim = dim3(P_THREADS);
     cfg.dynamicSmemBytes = t_smem_bytes<true>();
     cudaLaunchAttribute at[1];
@@ -609,14 +609,12 @@ static int pair_slots() {
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    int c = 0;
-    if (cudaOccupancyMaxActiveClusters(&c, k_gemm_tf32x3_t<true>, &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&l.pairs, k_gemm_tf32x3_t<true>, &cfg) != cudaSuccess) {
       (void)cudaGetLastError();
-      c = 0;
+      l.pairs = 0;
     }
-    n = c;
-  }
-  return n;
+    return l;
+  });
 }
 
 // Tile schedule of one product: CTA pairs (256-row tiles) whenever M spans more
@@ -628,9 +626,10 @@ struct Plan {
 };
 static Plan plan_of(int64_t M, int64_t N, int64_t K) {
   Plan p;
-  p.pair = M > BM && pair_slots() > 0;
+  const Limits lim = limits();
+  p.pair = M > BM && lim.pairs > 0;
   const int cs = p.pair ? 2 : 1;
-  p.slots = p.pair ? pair_slots() : sm_count();
+  p.slots = p.pair ? lim.pairs : lim.sms;
   p.mt = (M + BM * cs - 1) / (BM * cs);
   p.nt = (N + (p.pair ? t_bn<true>() : BN) - 1) / (p.pair ? t_bn<true>() : BN);
   const int64_t nk = (K + BK - 1) / BK;
@@ -650,12 +649,6 @@ void gemm_onchip(cudaStream_t s, int64_t M, int64_t N, int64_t K, const float* A
                  const Grading* graded, int mark) {
   FP_CHECK(scratch && scratch_bytes >= sizeof(int), FPEPS_ERR_ARG, "tensor-core GEMM: scratch");
   FP_CHECK(((uintptr_t)A % 16) == 0 && ((uintptr_t)B % 16) == 0, FPEPS_ERR_ARG, "tensor-core GEMM: operand alignment");
-  static bool attr = false;
-  if (!attr) {
-    FP_CUDA(cudaFuncSetAttribute(k_gemm_tf32x3_t<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 t_smem_bytes<false>()));
-    attr = true;
-  }
   const Plan p = plan_of(M, N, K);
   CUtensorMap ma = make_map(A, M, K, lda, BM);
   CUtensorMap mb = make_map(B, N, K, ldb, p.pair ? t_bn<true>() / 2 : BN);

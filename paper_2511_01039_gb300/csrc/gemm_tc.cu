@@ -632,24 +632,28 @@ CUtensorMap make_map(const __half* base, int64_t rows, int64_t nk, int box_rows)
   return m;
 }
 
-int sm_count() {
-  static int sms = 0;
-  if (!sms) {
-    int dev = 0;
-    FP_CUDA(cudaGetDevice(&dev));
-    FP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  }
-  return sms;
+// SMs, and CTA pairs the GPU holds at once (clusters of two CTAs, one CTA per SM; 0 if the pair kernel
+// cannot be launched). Asking for them also prepares the kernels for launches in this context.
+struct Limits {
+  int sms, pairs;
+};
+template <bool PAIR>
+void allow_smem() {
+  FP_CUDA(cudaFuncSetAttribute(k_gemm_f16x3<PAIR, ROWS_BULK>, cudaFuncAttributeMaxDynamicSharedMemorySize, t_smem_bytes<PAIR>()));
+  FP_CUDA(cudaFuncSetAttribute(k_gemm_f16x3<PAIR, ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize, t_smem_bytes<PAIR>()));
+  FP_CUDA(cudaFuncSetAttribute(k_gemm_f16x3<PAIR, LANES>, cudaFuncAttributeMaxDynamicSharedMemorySize, t_smem_bytes<PAIR>()));
 }
-
-// CTA pairs the GPU holds at once (clusters of two CTAs, one CTA per SM); 0 if the pair kernel
-// cannot be launched
-int pair_slots() {
-  static int n = -1;
-  if (n < 0) {
-    FP_CUDA(cudaFuncSetAttribute(k_gemm_f16x3<true, LANES>, cudaFuncAttributeMaxDynamicSharedMemorySize, t_smem_bytes<true>()));
+Limits limits() {
+  static PerContext<Limits> per;
+  return per.get([] {
+    allow_smem<false>();
+    allow_smem<true>();
+    int dev = 0;
+    Limits l{0, 0};
+    FP_CUDA(cudaGetDevice(&dev));
+    FP_CUDA(cudaDeviceGetAttribute(&l.sms, cudaDevAttrMultiProcessorCount, dev));
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(sm_count() & ~1));
+    cfg.gridDim = dim3((unsigned)(l.sms & ~1));
     cfg.blockDim = dim3(P_THREADS);
     cfg.dynamicSmemBytes = t_smem_bytes<true>();
     cudaLaunchAttribute at[1];
@@ -659,14 +663,12 @@ int pair_slots() {
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    int c = 0;
-    if (cudaOccupancyMaxActiveClusters(&c, k_gemm_f16x3<true, LANES>, &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&l.pairs, k_gemm_f16x3<true, LANES>, &cfg) != cudaSuccess) {
       (void)cudaGetLastError();
-      c = 0;
+      l.pairs = 0;
     }
-    n = c;
-  }
-  return n;
+    return l;
+  });
 }
 
 // Tile shape and schedule of one product: the estimated cycles of the busiest slot. A k-block costs
@@ -680,9 +682,10 @@ Plan plan_of(int64_t M, int64_t N, int64_t K) {
   Plan best;
   double cost = 1e300;
   const int64_t nk = (K + BK - 1) / BK, nch = (nk + CHB - 1) / CHB;
+  const Limits lim = limits();
   for (int pr = 0; pr < 2; ++pr) {
-    if (pr && (M <= BM || pair_slots() <= 0)) continue;
-    const int64_t most = pr ? pair_slots() : sm_count();
+    if (pr && (M <= BM || lim.pairs <= 0)) continue;
+    const int64_t most = pr ? lim.pairs : lim.sms;
     const int64_t mt = (M + BM * (1 + pr) - 1) / (BM * (1 + pr));
     for (int cap = BNMAX; cap >= 32; cap /= 2) {
       const int64_t w = (N + cap - 1) / cap;
@@ -716,10 +719,6 @@ Plan plan_of(int64_t M, int64_t N, int64_t K) {
 
 template <bool PAIR, int OUT>
 void launch_gemm(cudaStream_t s, int64_t slots, const CUtensorMap& ma, const CUtensorMap& mb, const TcArgs& g) {
-  static std::once_flag attr;
-  std::call_once(attr, [] {
-    FP_CUDA(cudaFuncSetAttribute(k_gemm_f16x3<PAIR, OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize, t_smem_bytes<PAIR>()));
-  });
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(slots * (PAIR ? 2 : 1)));
   cfg.blockDim = dim3(P_THREADS);

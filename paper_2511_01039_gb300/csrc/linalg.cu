@@ -702,14 +702,14 @@ void cholesky_inverse_f64(cudaStream_t s, double* G, double* X, int k, int* info
     k_chol_inv_small<<<1, 1024, (size_t)(k * (2 * k + 1) + k) * sizeof(double), s>>>(G, X, k, tol, info);
     FP_LAUNCH();
   } else {
-    static int max_blocks = -1;
-    if (max_blocks < 0) {
+    static PerContext<int> resident;
+    const int max_blocks = resident.get([] {
       int dev = 0, sms = 0, per = 0;
       FP_CUDA(cudaGetDevice(&dev));
       FP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
       FP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_chol_inv_coop, CH_NT, 0));
-      max_blocks = sms * std::max(per, 0);
-    }
+      return sms * std::max(per, 0);
+    });
     const int blocks = std::min(max_blocks, 152);
     FP_CHECK(blocks >= 1, FPEPS_ERR_CUDA, "cholesky: no co-resident blocks");
     void* args[] = {&G, &X, &k, &tol, &info};

@@ -531,19 +531,16 @@ void sandwich_apply_tc(cudaStream_t s, const SandOrient& o, int64_t nt, int64_t 
   const int nb_per = std::max(1, std::min(144 / K1, 144 / N2));
   const int64_t nblk = nt * nk;
   const int64_t ngroups = (nblk + nb_per - 1) / nb_per;
-  static int sms = 0;
-  if (sms == 0) {
-    int dev = 0;
-    FP_CUDA(cudaGetDevice(&dev));
-    FP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  }
-  const int64_t grid = std::min<int64_t>(ngroups, sms);
   const size_t smem = (size_t)SM_FLOATS * sizeof(float);
-  static bool attr = false;
-  if (!attr) {
+  static PerContext<int> per;   // SMs; the kernel is prepared with them
+  const int sms = per.get([&] {
     FP_CUDA(cudaFuncSetAttribute(k_sandwich_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    attr = true;
-  }
+    int dev = 0, n = 0;
+    FP_CUDA(cudaGetDevice(&dev));
+    FP_CUDA(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev));
+    return n;
+  });
+  const int64_t grid = std::min<int64_t>(ngroups, sms);
   k_sandwich_mma<<<(unsigned)grid, SM_THREADS, smem, s>>>(o, nt, nk, nb_per, ngroups, in, i_t, i_k, i_X, i_Y, out,
                                                           o_t, o_k, o_V, o_Z);
   FP_LAUNCH();
@@ -558,12 +555,11 @@ void sandwich_apply(cudaStream_t s, const SandOrient& o, int64_t nt, int64_t nk,
   size_t nacc = (size_t)o.nx * o.ny * o.nv * o.nz * o.p;
   size_t smem = (nsl + 3 * nacc) * sizeof(T);
   FP_CHECK(smem <= 200 * 1024, FPEPS_ERR_UNSUPPORTED, "sandwich: site too large for shared memory");
-  static bool attr_set[2] = {false, false};
-  int idx = sizeof(T) == 8 ? 1 : 0;
-  if (!attr_set[idx]) {
+  static PerContext<bool> prepared;
+  prepared.get([] {
     FP_CUDA(cudaFuncSetAttribute(k_sandwich<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-    attr_set[idx] = true;
-  }
+    return true;
+  });
   int64_t nblk = nt * nk;
   FP_CHECK(nblk < (1LL << 31), FPEPS_ERR_UNSUPPORTED, "sandwich: too many blocks");
   k_sandwich<T><<<(unsigned)nblk, 256, smem, s>>>(o, nk, in, i_t, i_k, i_X, i_Y, out, o_t, o_k, o_V, o_Z);

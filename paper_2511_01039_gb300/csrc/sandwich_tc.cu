@@ -731,17 +731,14 @@ void sandwich_apply_tcgen05(cudaStream_t s, const SandOrient& o, int64_t nt, int
   a.out = out; a.o_t = o_t; a.o_k = o_k; a.o_V = o_V; a.o_Z = o_Z;
   a.v_fast = o_V == 1 ? 1 : 0;   // the same rule as bundle_index's callers: V when it has unit stride
   a.err = err;
-  static int sms = 0;
-  if (sms == 0) {
-    int dev = 0;
-    FP_CUDA(cudaGetDevice(&dev));
-    FP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  }
-  static bool attr = false;
-  if (!attr) {
+  static PerContext<int> per;   // SMs; the kernel is prepared with them
+  const int sms = per.get([] {
     FP_CUDA(cudaFuncSetAttribute(k_sandwich_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SW_SMEM));
-    attr = true;
-  }
+    int dev = 0, n = 0;
+    FP_CUDA(cudaGetDevice(&dev));
+    FP_CUDA(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev));
+    return n;
+  });
   const int64_t grid = std::min<int64_t>(a.ngroups, sms);
   k_sandwich_tc<<<(unsigned)grid, SW_THREADS, SW_SMEM, s>>>(a);
   FP_LAUNCH();

@@ -746,11 +746,11 @@ void sweeps_f64(cudaStream_t s, double* Mat, int k, double* V, const int* skip, 
   // one CTA per pair of two-column blocks, all co-resident (cooperative launch)
   const int nb = (k + 1) / 2, blocks = (nb + (nb & 1)) / 2;
   const size_t smem = (8 * (size_t)k + 12) * sizeof(double), most = (8 * 1024 + 12) * sizeof(double);
-  static int max_blocks = -1;
-  if (max_blocks < 0) {
+  static PerContext<int> per;
+  const int max_blocks = per.get([&] {
     FP_CUDA(cudaFuncSetAttribute(k_jacobi_svd_blk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
-    max_blocks = resident(k_jacobi_svd_blk, JB_THREADS, most);
-  }
+    return resident(k_jacobi_svd_blk, JB_THREADS, most);
+  });
   FP_CHECK(blocks <= max_blocks, FPEPS_ERR_CUDA, "svd: too few co-resident blocks");
   unsigned long long* ws = (unsigned long long*)ws_dev;
   int max_sweeps = 30;
@@ -798,11 +798,11 @@ void svd_jacobi_f64(cudaStream_t s, double* Mat, int k, double* U, double* sigma
     k_svd_max<<<grid_of(kk), 256, 0, s>>>(Mat, kk, st);
     FP_LAUNCH();
     if (k <= J32_ONE) {
-      static bool attr = false;
-      if (!attr) {
+      static PerContext<bool> prepared;
+      prepared.get([] {
         FP_CUDA(cudaFuncSetAttribute(k_jacobi32, cudaFuncAttributeMaxDynamicSharedMemorySize, (3 * J32_ONE * (J32_ONE + 1) + J32_ONE) * 4));
-        attr = true;
-      }
+        return true;
+      });
       k_jacobi32<<<1, 32 * std::min(32, (k + 1) / 2), (size_t)(3 * k * (k | 1) + k) * 4, s>>>(Mat, k, st, T1);
       FP_LAUNCH();
     } else {
@@ -811,12 +811,12 @@ void svd_jacobi_f64(cudaStream_t s, double* Mat, int k, double* U, double* sigma
         const int rows = (n + grid - m_ctas - 1) / (grid - m_ctas);
         return (size_t)std::max(2 * J32_B * (n | 1) + 2 * J32_B, 2 * rows * (n | 1)) * 4;
       };
-      static int max_blocks = -1;
-      if (max_blocks < 0) {   // the largest need: 1024 columns on 64 + 64 CTAs
+      static PerContext<int> per;
+      const int max_blocks = per.get([&] {   // the largest need: 1024 columns on 64 + 64 CTAs
         const size_t most = smem_of(1024, 128, 64);
         FP_CUDA(cudaFuncSetAttribute(k_jacobi32_blk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
-        max_blocks = std::min(resident(k_jacobi32_blk, 32 * J32_B, most), 152);
-      }
+        return std::min(resident(k_jacobi32_blk, 32 * J32_B, most), 152);
+      });
       FP_CHECK(max_blocks >= 2 * nm, FPEPS_ERR_CUDA, "svd: too few co-resident blocks");
       const int blocks = std::min(max_blocks, nm + k);
       J32Args g;

@@ -14,15 +14,11 @@
 // ordering, counters and norms, for k <= FPEPS_SVD_NOALLOC_MAX_K (256), about 3 MB. Every GPU that loads the
 // library holds it until the process exits. In host code the symbol names a
 // host-side stand-in, not device memory, so it is never handed to a kernel
-// directly: on the first call on a device (with that device current) its device
-// address is looked up once with cudaGetSymbolAddress and cached; later calls
-// on that device reuse it. The cached address belongs to the device's primary
-// context: after cudaDeviceReset (which destroys that context) it is stale, so a
-// process that resets a device must not call this entry point on it again. All
-// calls share the array: calls whose work overlaps on the GPU (different streams,
+// directly: on the first call in a context its device address is looked up with
+// cudaGetSymbolAddress and kept for the later calls there (a context that follows
+// a cudaDeviceReset looks it up again). All calls share the array: calls whose work overlaps on the GPU (different streams,
 // or different host threads) race on it.
 #include <exception>
-#include <mutex>
 
 #include "common.cuh"
 
@@ -35,22 +31,15 @@ constexpr size_t kScratchBytes = 5 * (size_t)kMaxK * kMaxK * sizeof(double) + ((
                                  (size_t)kMaxK * (sizeof(int) + sizeof(double)) + 4096;
 static __device__ __align__(256) unsigned char g_svd_scratch[kScratchBytes];
 
-std::mutex g_mu;
-void* g_addr[64] = {};
-
-// device address of g_svd_scratch on the current device (looked up once per device)
+// device address of g_svd_scratch in the current context (looked up once)
 char* scratch_address() {
-  int dev = 0;
-  FP_CUDA(cudaGetDevice(&dev));
-  FP_CHECK(dev >= 0 && dev < 64, FPEPS_ERR_UNSUPPORTED, "device index out of range");
-  std::lock_guard<std::mutex> lk(g_mu);
-  if (!g_addr[dev]) {
+  static PerContext<char*> per;
+  return per.get([] {
     void* p = nullptr;
     FP_CUDA(cudaGetSymbolAddress(&p, g_svd_scratch));
     FP_CHECK(p != nullptr, FPEPS_ERR_CUDA, "cudaGetSymbolAddress returned NULL");
-    g_addr[dev] = p;
-  }
-  return static_cast<char*>(g_addr[dev]);
+    return static_cast<char*>(p);
+  });
 }
 
 }  // namespace
