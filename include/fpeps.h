@@ -331,7 +331,10 @@ fpeps_status fpeps_apply_theta_op(fpeps_env* env, int32_t op, int32_t c, int32_t
  * mode FPEPS_F32: CUDA-core FP32; FPEPS_TF32X3 / FPEPS_BF16X3: 22-bit split
  * products on the tensor cores (needs K >= 32, lda and ldb multiples of 4, 16-byte aligned
  * A and B, else FPEPS_ERR_UNSUPPORTED). Synchronises `cuda_stream` for the
- * tensor-core modes. */
+ * tensor-core modes, which take their scratch stream-ordered from a pool of the
+ * library: about half a gigabyte for the split copies of a large product, or
+ * 8 KB x (M + N) where that is more, and less where there is no room. The pool
+ * keeps up to 640 MB (see fpeps_release_scratch). */
 fpeps_status fpeps_gemm_f32(int32_t mode, int64_t M, int64_t N, int64_t K, const float* A, int64_t lda,
                             const float* B, int64_t ldb, float* C, void* cuda_stream);
 
@@ -344,8 +347,8 @@ fpeps_status fpeps_gemm_f32(int32_t mode, int64_t M, int64_t N, int64_t K, const
  * checked in FP64); the sweep count is capped at 30, so a badly conditioned
  * general matrix may return before full convergence. A NaN or an infinity in M
  * comes back as NaN or infinite singular values.
- * Takes its scratch (about 5.5 k^2 doubles) stream-ordered on `cuda_stream` from a
- * pool of the library, and synchronises the stream. */
+ * Takes its scratch (about 5.5 k^2 doubles) stream-ordered on `cuda_stream` from the
+ * same pool as fpeps_gemm_f32, and synchronises the stream. */
 fpeps_status fpeps_svd_f64(const double* M, int32_t k, double* U, double* sigma, double* V, void* cuda_stream);
 
 /* Largest k accepted by fpeps_svd_f64_noalloc. */
@@ -377,6 +380,12 @@ fpeps_status fpeps_svd_f64_noalloc(const double* M, int32_t k, double* U, double
  * cudaMallocAsync on `cuda_stream` and synchronises it. The paper has no
  * counterpart. */
 fpeps_status fpeps_selftest_wait_timeout(void* cuda_stream);
+
+/* Gives back the device memory that fpeps_gemm_f32 and fpeps_svd_f64 keep in the current
+ * context from one call to the next (at most 640 MB), after a wait for the device. An
+ * allocation of the library that fails does the same before it is tried again; destroying
+ * an environment gives back what is free by then. */
+fpeps_status fpeps_release_scratch(void);
 
 /* Number of kernels this library has launched in the process so far. */
 int64_t fpeps_launch_count(void);

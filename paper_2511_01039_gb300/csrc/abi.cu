@@ -44,14 +44,14 @@ uint64_t context_id() {
 // Scratch of the calls without a handle (fpeps_gemm_f32): a pool of the library's own per context,
 // shared by all threads and streams (stream-ordered). The default pool hands its memory back at
 // every synchronisation, and mapping half a gigabyte again costs the next call a millisecond; this
-// one keeps up to kKeep bytes, which trim_pool() gives back (when an environment is destroyed or an
-// allocation fails).
+// one keeps up to kKeep bytes, which trim_pool() gives back (when an environment is destroyed, an
+// allocation fails, or the caller asks).
 namespace {
 constexpr uint64_t kKeep = 640ull << 20;
 PerContext<cudaMemPool_t> g_pools;
 }  // namespace
 
-static cudaMemPool_t scratch_pool() {
+static cudaMemPool_t scratch_pool(uint64_t context) {
   return g_pools.get([] {
     int dev = 0;
     FP_CUDA(cudaGetDevice(&dev));
@@ -64,7 +64,7 @@ static cudaMemPool_t scratch_pool() {
     uint64_t keep = kKeep;
     FP_CUDA(cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep));
     return pool;
-  });
+  }, context);
 }
 
 // Pinned words for the status that a call without a handle reads back, one set per thread and context:
@@ -73,15 +73,15 @@ static cudaMemPool_t scratch_pool() {
 struct StatusWords {
   static constexpr int N = 8;   // error word, grading (kTcHeader's first words)
   std::map<uint64_t, int*> words;
-  int* get() {
-    auto it = words.find(context_id());
+  int* get(uint64_t context) {
+    auto it = words.find(context);
     if (it != words.end()) return it->second;
     int* p = nullptr;
     if (cudaHostAlloc((void**)&p, N * sizeof(int), cudaHostAllocDefault) != cudaSuccess) {
       cudaGetLastError();
       return nullptr;
     }
-    return words[context_id()] = p;
+    return words[context] = p;
   }
   ~StatusWords() {   // the current context's; another one's may be gone, with its words
     try {
@@ -94,10 +94,13 @@ struct StatusWords {
   }
 };
 
-// the scratch pool of the current context
-static void trim_pool() {
+// What the scratch pool of the current context keeps goes back to the device. wait: also what the last
+// calls freed, stream-ordered, without a wait after it.
+static void trim_pool(bool wait) {
   cudaMemPool_t pool;
-  if (g_pools.peek(pool)) cudaMemPoolTrimTo(pool, 0);
+  if (!g_pools.peek(pool)) return;
+  if (wait) FP_CUDA(cudaDeviceSynchronize());
+  cudaMemPoolTrimTo(pool, 0);
 }
 
 void* Allocator::get(size_t bytes) {
@@ -105,7 +108,7 @@ void* Allocator::get(size_t bytes) {
   if (has) {
     p = a.alloc(a.ctx, bytes, (void*)stream);
     if (!p) {
-      trim_pool();
+      trim_pool(true);
       if (reclaim) reclaim();
       p = a.alloc(a.ctx, bytes, (void*)stream);
     }
@@ -115,7 +118,7 @@ void* Allocator::get(size_t bytes) {
   cudaError_t e = cudaMallocAsync(&p, bytes, stream);
   if (e == cudaErrorMemoryAllocation) {
     cudaGetLastError();
-    trim_pool();
+    trim_pool(true);
     if (reclaim) reclaim();
     e = cudaMallocAsync(&p, bytes, stream);
   }
@@ -687,7 +690,7 @@ void fpeps_env_destroy(fpeps_env* env) {
     if (env->stream || !env->al.has) cudaStreamSynchronize(env->stream);
     if (env->h_info) cudaFreeHost(env->h_info);
     if (env->h_scal) cudaFreeHost(env->h_scal);
-    fpeps::trim_pool();
+    fpeps::trim_pool(false);
   } catch (...) {
   }
   delete env;
@@ -786,29 +789,37 @@ fpeps_status fpeps_gemm_f32(int32_t mode, int64_t M, int64_t N, int64_t K, const
       throw Error{FPEPS_ERR_UNSUPPORTED, "shape not supported by the tensor-core kernel"};
     size_t sb = fpeps::gemm_tc_scratch_bytes(M, N, K);
     int* err = nullptr;
-    cudaError_t e = cudaMallocFromPoolAsync((void**)&err, sb, fpeps::scratch_pool(), s);
+    const uint64_t context = fpeps::context_id();
+    const cudaMemPool_t pool = fpeps::scratch_pool(context);
+    cudaError_t e = cudaMallocFromPoolAsync((void**)&err, sb, pool, s);
     if (e == cudaErrorMemoryAllocation) {   // no room for planes: the on-chip split needs little
       cudaGetLastError();
       sb = fpeps::gemm_onchip_scratch_bytes(M, N, K);
-      e = cudaMallocFromPoolAsync((void**)&err, sb, fpeps::scratch_pool(), s);
+      e = cudaMallocFromPoolAsync((void**)&err, sb, pool, s);
     }
     FP_CUDA(e);
     FP_CUDA(cudaMemsetAsync(err, 0, fpeps::kTcHeader, s));
     fpeps::gemm_tc(s, M, N, K, A, lda, B, ldb, C, om, err, sb, 1, false);
     static thread_local fpeps::StatusWords words;
     int on_stack[fpeps::StatusWords::N] = {};
-    int* const pinned = words.get();
+    int* const pinned = words.get(context);
     int* const h = pinned ? pinned : on_stack;
-    FP_CUDA(cudaMemcpyAsync(h, err, sizeof(on_stack), cudaMemcpyDeviceToHost, s));
-    FP_CUDA(cudaStreamSynchronize(s));
+    auto status = [&] {
+      FP_CUDA(cudaMemcpyAsync(h, err, sizeof(on_stack), cudaMemcpyDeviceToHost, s));
+      FP_CUDA(cudaStreamSynchronize(s));
+    };
+    status();
     if (!*h && (h[4] || h[5] || h[6])) {   // deep or narrow segments: the rest of the test, and the on-chip split if graded
       fpeps::gemm_tc_settle(s, M, N, K, A, lda, B, ldb, C, om, err, sb, 1);
-      FP_CUDA(cudaMemcpyAsync(h, err, sizeof(int), cudaMemcpyDeviceToHost, s));
-      FP_CUDA(cudaStreamSynchronize(s));
+      status();
     }
-    cudaFreeAsync(err, s);
+    FP_CUDA(cudaFreeAsync(err, s));   // (before the wait it adds 2 us to a call)
     if (*h) throw Error{FPEPS_ERR_TIMEOUT, "tensor-core GEMM timed out"};
   });
+}
+
+fpeps_status fpeps_release_scratch(void) {
+  return fpeps::guard(nullptr, [] { fpeps::trim_pool(true); });
 }
 
 fpeps_status fpeps_svd_f64(const double* M, int32_t k, double* U, double* sigma, double* V, void* cuda_stream) {
@@ -819,7 +830,7 @@ fpeps_status fpeps_svd_f64(const double* M, int32_t k, double* U, double* sigma,
     char* scr = nullptr;
     auto up = [](size_t n) { return (n + 255) / 256 * 256; };
     const size_t b_mat = up(2 * kk * sizeof(double)), b_ord = up((size_t)k * sizeof(int)), b_ws = up(fpeps::svd_ws_bytes(k));
-    FP_CUDA(cudaMallocFromPoolAsync((void**)&scr, b_mat + b_ord + b_ws + std::max<size_t>(fpeps::svd_work_bytes(k), 16), fpeps::scratch_pool(), s));
+    FP_CUDA(cudaMallocFromPoolAsync((void**)&scr, b_mat + b_ord + b_ws + std::max<size_t>(fpeps::svd_work_bytes(k), 16), fpeps::scratch_pool(fpeps::context_id()), s));
     double* Mw = (double*)scr;
     double* Vw = Mw + kk;
     int* order = (int*)(scr + b_mat);

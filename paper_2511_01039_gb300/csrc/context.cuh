@@ -18,8 +18,7 @@ template <class T>
 class PerContext {
  public:
   template <class Make>
-  T get(Make&& make) {
-    const uint64_t id = context_id();
+  T get(Make&& make, uint64_t id = context_id()) {
     std::lock_guard<std::mutex> lk(mu_);
     auto it = made_.find(id);
     if (it == made_.end()) it = made_.emplace(id, make()).first;

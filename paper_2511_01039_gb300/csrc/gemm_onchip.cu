@@ -639,17 +639,17 @@ static Plan plan_of(int64_t M, int64_t N, int64_t K) {
   return p;
 }
 
-size_t gemm_onchip_scratch_bytes(int64_t M, int64_t N, int64_t K) {
-  const Plan p = plan_of(M, N, K);
-  return 256 + (p.nsplit > 1 ? (size_t)p.nsplit * M * N * sizeof(float) : 0);
+static size_t scratch_of(const Plan& p, int64_t M, int64_t N) {
+  return kTcHeader + (p.nsplit > 1 ? (size_t)p.nsplit * M * N * sizeof(float) : 0);
 }
+size_t gemm_onchip_scratch_bytes(int64_t M, int64_t N, int64_t K) { return scratch_of(plan_of(M, N, K), M, N); }
 
 void gemm_onchip(cudaStream_t s, int64_t M, int64_t N, int64_t K, const float* A, int64_t lda, const float* B,
                  int64_t ldb, float* C, OutMap om, void* scratch, size_t scratch_bytes, bool hold_loads,
                  const Grading* graded, int mark) {
-  FP_CHECK(scratch && scratch_bytes >= sizeof(int), FPEPS_ERR_ARG, "tensor-core GEMM: scratch");
   FP_CHECK(((uintptr_t)A % 16) == 0 && ((uintptr_t)B % 16) == 0, FPEPS_ERR_ARG, "tensor-core GEMM: operand alignment");
   const Plan p = plan_of(M, N, K);
+  FP_CHECK(scratch && scratch_bytes >= scratch_of(p, M, N), FPEPS_ERR_ARG, "tensor-core GEMM: scratch too small");
   CUtensorMap ma = make_map(A, M, K, lda, BM);
   CUtensorMap mb = make_map(B, N, K, ldb, p.pair ? t_bn<true>() / 2 : BN);
   TcArgs g;
@@ -666,8 +666,7 @@ void gemm_onchip(cudaStream_t s, int64_t M, int64_t N, int64_t K, const float* A
   g.mark = mark;
   g.part = nullptr;
   if (g.nsplit > 1) {
-    FP_CHECK(scratch_bytes >= gemm_onchip_scratch_bytes(M, N, K), FPEPS_ERR_ARG, "tensor-core GEMM: scratch too small");
-    g.part = (float*)((char*)scratch + 256);
+    g.part = (float*)((char*)scratch + kTcHeader);
   }
   const int64_t tiles = g.mt * g.nt * g.nsplit;
   FP_CHECK(tiles < (1LL << 30), FPEPS_ERR_UNSUPPORTED, "tensor-core GEMM: grid too large");

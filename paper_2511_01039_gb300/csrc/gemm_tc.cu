@@ -821,7 +821,6 @@ size_t gemm_tc_scratch_bytes(int64_t M, int64_t N, int64_t K) {
 void gemm_tc(cudaStream_t s, int64_t M, int64_t N, int64_t K, const float* A, int64_t lda, const float* B,
              int64_t ldb, float* C, OutMap om, void* scratch, size_t scratch_bytes, int mark, bool settle) {
   FP_CHECK(((uintptr_t)A % 16) == 0 && ((uintptr_t)B % 16) == 0, FPEPS_ERR_ARG, "tensor-core GEMM: operand alignment");
-  FP_CHECK(scratch && scratch_bytes >= gemm_onchip_scratch_bytes(M, N, K), FPEPS_ERR_ARG, "tensor-core GEMM: scratch too small");
   ProfToken pt = prof_begin(PROF_GEMM_TC, s, 2.0 * M * N * K, 4.0 * ((double)M * K + (double)N * K + (double)M * N));
   if (!on_planes(M, N, K) || scratch_bytes < gemm_tc_scratch_bytes(M, N, K)) {
     gemm_onchip(s, M, N, K, A, lda, B, ldb, C, om, scratch, scratch_bytes);

@@ -83,6 +83,7 @@ SIGNATURES = {
                                  C.c_int64, C.c_void_p, C.c_void_p]),
     "fpeps_svd_f64": (C.c_int, [C.c_void_p, C.c_int32, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p]),
     "fpeps_svd_f64_noalloc": (C.c_int, [C.c_void_p, C.c_int32, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p]),
+    "fpeps_release_scratch": (C.c_int, []),
     "fpeps_launch_count": (C.c_int64, []),
     "fpeps_selftest_wait_timeout": (C.c_int, [C.c_void_p]),
     "fpeps_profile": (C.c_int, [C.c_int32]),
@@ -305,6 +306,11 @@ def fpeps_svd_f64_noalloc(M, stream_handle: int = 0):
     _check(None, lib().fpeps_svd_f64_noalloc(Mc.data_ptr(), k, U.data_ptr(), s.data_ptr(), V.data_ptr(),
                                              stream_handle))
     return U.t(), s, V.t()
+
+
+def fpeps_release_scratch():
+    """Give back the device memory that fpeps_gemm_f32 and fpeps_svd_f64 keep between calls."""
+    _check(None, lib().fpeps_release_scratch())
 
 
 PROF_KINDS = {0: "gemm_tc_tf32x3", 1: "gemm_simt", 2: "sandwich", 3: "gram", 4: "factor", 5: "sketch"}

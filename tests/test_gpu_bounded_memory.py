@@ -138,3 +138,20 @@ def test_refused_growth_leaves_the_handle_usable():
     assert al.refused and al.stray == 0
     fp.fpeps_env_destroy(h)
     assert al.stray == 0 and not al.live
+
+
+def test_scratch_of_calls_without_a_handle_is_given_back():
+    """A large product leaves its scratch with the library (at most 640 MB) until the caller asks for it."""
+    import torch
+    from paper_2511_01039_gb300 import fpeps as fp
+    A, B, C = (torch.ones(s, device="cuda") for s in ((500, 40000), (8000, 40000), (500, 8000)))
+    fp.fpeps_release_scratch()
+    torch.cuda.synchronize()
+    start = torch.cuda.mem_get_info()[0]
+    fp.fpeps_gemm_f32(fp.TF32X3, A, B, C)
+    kept = start - torch.cuda.mem_get_info()[0]
+    assert kept <= 700 << 20
+    fp.fpeps_release_scratch()
+    assert start - torch.cuda.mem_get_info()[0] <= 32 << 20 < kept
+    fp.fpeps_gemm_f32(fp.TF32X3, A, B, C)
+    assert (C == 40000).all()
