@@ -95,7 +95,8 @@ inline OutMap out_colmajor(int64_t M, int64_t N, int64_t ldc) { return OutMap{M,
 template <class T>
 void gemm_simt(cudaStream_t s, int64_t M, int64_t N, int64_t K, T alpha, const T* A, int64_t a_m,
                int64_t a_k, const T* B, int64_t b_n, int64_t b_k, T beta, T* C, OutMap om,
-               const int* skip = nullptr);   // device flag: nothing is done when it is set
+               const int* skip = nullptr,    // device flag: nothing is done when it is set
+               bool record = true);          // false: part of a step that has a profile record of its own
 
 // Tensor-core GEMM for K-major A [M][lda] and B [N][ldb] (k contiguous), every operand split
 // into two 11-bit halves: products that amortise it run on FP16 planes made beforehand (gemm_tc.cu),

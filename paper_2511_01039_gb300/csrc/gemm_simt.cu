@@ -367,12 +367,13 @@ void run_big(cudaStream_t s, int split, int64_t M, int64_t N, int64_t K, float a
 
 template <class T>
 void gemm_simt(cudaStream_t s, int64_t M, int64_t N, int64_t K, T alpha, const T* A, int64_t a_m, int64_t a_k,
-               const T* B, int64_t b_n, int64_t b_k, T beta, T* C, OutMap om, const int* skip) {
+               const T* B, int64_t b_n, int64_t b_k, T beta, T* C, OutMap om, const int* skip, bool record) {
   if (M <= 0 || N <= 0) return;
   FP_CHECK(om.mdiv > 0 && om.ndiv > 0, FPEPS_ERR_ARG, "gemm: bad output map");
   FP_CHECK((M + 63) / 64 <= 65535, FPEPS_ERR_UNSUPPORTED, "gemm: M too large for grid");
-  ProfToken pt = prof_begin(PROF_GEMM_SIMT, s, 2.0 * M * N * K,
-                            (double)sizeof(T) * ((double)M * K + (double)N * K + (double)M * N));
+  ProfToken pt;
+  if (record)
+    pt = prof_begin(PROF_GEMM_SIMT, s, 2.0 * M * N * K, (double)sizeof(T) * ((double)M * K + (double)N * K + (double)M * N));
   const Pick p = pick(M, N, K, sizeof(T) == 8, b_k == 1);
   auto go = [&](auto run) { run(s, p.split, M, N, K, alpha, A, a_m, a_k, B, b_n, b_k, beta, C, om, skip); };
   if (p.kind == 0) go(run_tile<T, 64, 16>);
@@ -388,8 +389,8 @@ void gemm_simt(cudaStream_t s, int64_t M, int64_t N, int64_t K, T alpha, const T
 }
 
 template void gemm_simt<float>(cudaStream_t, int64_t, int64_t, int64_t, float, const float*, int64_t, int64_t,
-                               const float*, int64_t, int64_t, float, float*, OutMap, const int*);
+                               const float*, int64_t, int64_t, float, float*, OutMap, const int*, bool);
 template void gemm_simt<double>(cudaStream_t, int64_t, int64_t, int64_t, double, const double*, int64_t, int64_t,
-                                const double*, int64_t, int64_t, double, double*, OutMap, const int*);
+                                const double*, int64_t, int64_t, double, double*, OutMap, const int*, bool);
 
 }  // namespace fpeps

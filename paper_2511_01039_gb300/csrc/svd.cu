@@ -834,7 +834,7 @@ void svd_jacobi_f64(cudaStream_t s, double* Mat, int k, double* U, double* sigma
     }
     // column-major C = A B (or A^T B), optionally skipped or added to
     auto mul = [&](const double* A, bool ta, const double* B, double* C, double beta, const int* skip) {
-      gemm_simt<double>(s, k, k, k, 1.0, A, ta ? k : 1, ta ? 1 : k, B, k, 1, beta, C, out_colmajor(k, k, k), skip);
+      gemm_simt<double>(s, k, k, k, 1.0, A, ta ? k : 1, ta ? 1 : k, B, k, 1, beta, C, out_colmajor(k, k, k), skip, false);
     };
     mul(T1, true, T1, T2, 0.0, nullptr);
     k_svd_schulz<<<grid_of(kk), 256, 0, s>>>(T2, Mat, k, st);
