@@ -12,6 +12,7 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "rsqrt.cuh"
 
 namespace fpeps {
 namespace {
@@ -212,21 +213,6 @@ __global__ void __launch_bounds__(256, 2) k_gram_df(const float* __restrict__ Y,
 // elimination runs on [G | I]. A pivot at or below tol * max diag means column j depends
 // numerically on the columns before it: row j of R is set to zero (the column of Q it would give
 // is zero), and with it row and column j of X. info[0] |= 1 for non-finite input.
-//
-// 1 / sqrt(x) from the FP32 value by one step of Householder's third-order iteration (the Taylor
-// series of (1 - r)^(-1/2), r = 1 - x y^2 ~ 2^-22): about 320 cycles of dependent FP64 operations, half
-// of what rsqrt() takes here, on the critical path of every column.
-__device__ __forceinline__ double rsqrt_fast(double x) {
-  const int hi = __double2hiint(x);
-  if (hi < 0x00100000) return rsqrt(x);   // below the normal range
-  const int e = ((hi >> 20) - 1023) & ~1;
-  const double m = __hiloint2double(hi - (e << 20), __double2loint(x));   // [1, 4)
-  const double y = (double)rsqrtf((float)m);
-  const double r = fma(-(m * y), y, 1.0);
-  const double p = fma(fma(r, 0.3125, 0.375), r, 0.5);
-  const double z = fma(p, y * r, y);
-  return __hiloint2double(__double2hiint(z) - ((e / 2) << 20), __double2loint(z));
-}
 
 // The elimination of the n columns of D = [A | I] (shared memory, rows of ld doubles, A in columns 0 ..
 // n - 1, I in n .. 2 n - 1) by one CTA of NT threads; n <= 48. Warp 0 takes
