@@ -88,3 +88,28 @@ def test_patterns_of_large_and_small_terms(kind):
         A[:, k % 256 > 60] = 0
         B[:, k % 7 > 2] = 0
     assert _worst(_product(A, B, K), A, B) < 4e-6
+
+
+def test_site_map_of_graded_vectors():
+    """Theta^T sums over the environment's row index: powers of two on the rows of the environment, their
+    inverses on the vectors, leave the map as it is. Tolerance: two maps, each of two split products and
+    the sandwich, 4e-6 of sum |a b|, at most 16 times the largest output of N(0,1) data."""
+    import numpy as np
+    from paper_2511_01039_gb300 import fpeps as fp
+    from paper_2511_01039_gb300 import workloads as WL
+    from synth import lattice as L
+    D, w, chi, k = 6, 4, 500, 30
+    b = D * w * D
+    env = fp.Env(L.random_peps(3, 3, D, 4, seed=2), L.fsm_pepo(L.random_hamiltonian(3, 3, 4, w - 2, 2)), D=D, p=4, w=w, chi=chi,
+                 prec="tf32x3", seed=1)
+    g = np.random.default_rng(3)
+    bnd = [g.standard_normal(s, dtype=np.float32) for s in ((1, b, chi), (chi, b, chi), (chi, b, 1))]
+    fp.fpeps_import_boundary(env.h, WL.boundary_blob(bnd, 1, 1, 4), 1, 1)
+    fp.fpeps_absorb_row(env.h, 1, 1)
+    e = g.standard_normal((chi, chi, b), dtype=np.float32)
+    x = g.standard_normal((k, chi, b), dtype=np.float32)
+    f = np.exp2(-((np.arange(chi) % 250) * 36 // 250)).astype(np.float32)[:, None, None]
+    plain = env.apply_theta_op(1, 1, e, x, (chi, b))
+    graded = env.apply_theta_op(1, 1, e * f, x / f[None, :, :, 0], (chi, b))
+    env.close()
+    assert np.abs(graded - plain).max() < 2 * 3 * 16 * 4e-6 * np.abs(plain).max()
