@@ -165,7 +165,8 @@ __global__ void __launch_bounds__(256) k_uneven(SplitOp a, SplitOp b, int64_t K,
   const int64_t wa = a.rows * (int64_t)nseg, tot = wa + b.rows * (int64_t)nseg;
   for (int64_t w = blockIdx.x * (int64_t)(blockDim.x / 32) + threadIdx.x / 32; w < tot; w += (int64_t)gridDim.x * (blockDim.x / 32)) {
     const int which = w < wa ? 0 : 1;
-    if (!need[which] || *(volatile int*)&gr->uneven[which] == mark) continue;
+    // voted: other warps raise the word meanwhile, and all lanes take part in the reductions below
+    if (__any_sync(0xffffffffu, !need[which] || *(volatile int*)&gr->uneven[which] == mark)) continue;
     const SplitOp& o = which ? b : a;
     const int64_t v = which ? w - wa : w, row = v / nseg, seg = v % nseg;
     const int len = (int)min((int64_t)SEG, K - seg * SEG);
