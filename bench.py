@@ -196,17 +196,16 @@ def roofline_of(kind: str, d: dict, prec: str, peaks: dict) -> dict:
     intensity = d["flops"] / d["bytes"] if d["bytes"] > 0 else float("inf")   # flop per byte
     tensor_kinds = ("gemm_tc_tf32x3", "sandwich") if prec in ("tf32x3", "bf16x3") else ("gemm_tc_tf32x3",)
     if kind in tensor_kinds:
-        # bf16x3 GEMMs against the BF16 peak; tf32x3 (and the sandwich in either mode) against the
-        # TF32 dense peak = BF16 x nominal TF32/BF16 ratio
-        bfk = prec == "bf16x3" and kind == "gemm_tc_tf32x3"
-        peak = bf16 if bfk else bf16 * 1.1 / 2.25
+        # Peak: TF32 dense = BF16 x nominal TF32/BF16 ratio. Ceiling: what three MMAs per product leave, of
+        # the TF32 rate for the sandwich, of the BF16 rate for the GEMMs (most run on FP16 planes)
+        peak = bf16 * 1.1 / 2.25
+        ceiling = (bf16 if kind == "gemm_tc_tf32x3" else peak) / 3.0
         ridge = (peak / 3.0) * 1e12 / (hbm * 1e9)
         if intensity >= ridge:
-            what = f"BF16 peak {src}" if bfk else f"TF32 peak = {src} BF16 x 1.1/2.25"
             return {"bound": "tensor", "achieved": tflops, "peak": peak, "unit": "TFLOP/s", "frac": tflops / peak,
-                    "traffic": traffic, "kernel": kind,
-                    "note": f"{what}; algorithmic flops, and a 3-way split issues 3 MMAs per product: most GEMMs "
-                            f"run on FP16 planes, whose ceiling is BF16 peak / 3 = {bf16 / 3:.0f} TFLOP/s"}
+                    "ceiling": ceiling, "frac_of_ceiling": tflops / ceiling, "traffic": traffic, "kernel": kind,
+                    "note": f"peak: TF32 = {src} BF16 x 1.1/2.25; algorithmic flops, and a split product issues three "
+                            f"MMAs, FP16 ones in the GEMMs: the ceiling is a third of the rate they run at"}
         return {"bound": "hbm", "achieved": gbs, "peak": hbm, "unit": "GB/s", "frac": gbs / hbm, "traffic": traffic,
                 "kernel": kind,
                 "note": f"{intensity:.1f} algorithmic flop/byte, below the 3xTF32 ridge of {ridge:.1f} flop/byte "

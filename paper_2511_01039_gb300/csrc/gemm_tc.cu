@@ -40,7 +40,7 @@
 // What bounds it: 3 MMAs per term at the tensor rate (631 TFLOP/s, a third of the measured BF16
 // rate) for long sums, the epilogue and the power limit otherwise. Measured on GB300, splitting pass
 // included, on-chip TF32 split -> this: 8192 x 8192 x 8192 4.06 -> 2.19 ms (502 TFLOP/s), 108000 x
-// 9936 x 500 4.32 -> 2.38 ms, 108000 x 1728 x 500 0.79 -> 0.52 ms, 500 x 9936 x 108000 4.41 ->
+// 9936 x 500 4.32 -> 2.38 ms, 108000 x 1728 x 500 0.79 -> 0.54 ms, 500 x 9936 x 108000 4.41 ->
 // 3.66 ms (a third of it the splitting pass over 4.3 GB of B). The mainloop alone reaches 600
 // TFLOP/s at K = 500. Error against FP64 on N(0,1) data 9.4e-7 (on-chip TF32 1.8e-6: an FP16 MMA
 // adds twice the terms per truncating accumulation).
