@@ -60,10 +60,11 @@ typedef enum {
  * split into TF32 halves on chip; large ones into FP16 halves with a power-of-two
  * scale per row and 256 terms, where an element more than 2^17 below the largest
  * of its row and 256 terms keeps 2^-39 of that largest instead. Where such elements
- * can carry a sum (operands graded against each other along it), a large product is
- * split on chip too. BF16X3 (two
- * 8-bit halves, 3 x 2^-16) is at most as accurate as that and no faster, so a
- * BF16X3 environment runs the same products. The site sandwich is 3xTF32, and the
+ * can carry a sum (operands graded against each other along it: looked for in the QR
+ * and SVD steps, in maps of a caller's vectors and in fpeps_gemm_f32), a large product
+ * is split on chip too. BF16X3 (two 8-bit halves, 3 x 2^-16) runs the same products:
+ * halves of its own would be less accurate, no faster in the large ones and 7 % faster
+ * in those split on chip. The site sandwich is 3xTF32, and the
  * calibration columns and unbiased products run on the FP32 CUDA cores. */
 typedef enum { FPEPS_F64 = 0, FPEPS_F32 = 1, FPEPS_TF32X3 = 2, FPEPS_BF16X3 = 3 } fpeps_precision;
 
